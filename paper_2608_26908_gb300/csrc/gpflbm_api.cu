@@ -395,6 +395,9 @@ void set_device_params(gpflbm_t h) {
     }
     h->inv.inv2A[a] = 1.0 / (2.0 * h->params.A[a]);
   }
+  h->inv.same_A = 1;
+  for (int a = 1; a < h->NP; ++a)
+    if (h->inv.inv2A[a] != h->inv.inv2A[0]) h->inv.same_A = 0;
 }
 
 const void* dev_params(gpflbm_t h) {

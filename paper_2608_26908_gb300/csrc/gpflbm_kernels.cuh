@@ -822,6 +822,7 @@ struct InvParams {
   double theta_t, G;
   long long vlayer;
   int tdep;
+  int same_A;  // every phase of the problem has the same A (inv2A)
 };
 
 constexpr int kRedThreads = 256;
@@ -846,89 +847,276 @@ __device__ __forceinline__ double warp_sum_butterfly(double v) {
   return v;
 }
 
+// (double)x by integer arithmetic: GB300 converts on its FP64 pipe, one warp
+// instruction every 16 cycles an SM.  (A zero of either sign gives +0.)
+__device__ __forceinline__ double widen(double x) { return x; }
+__device__ __forceinline__ double widen(float x) {
+  const unsigned b = __float_as_uint(x);
+  double r = __hiloint2double((int)((b & 0x80000000u) | (((b & 0x7fffffffu) >> 3) + 0x38000000u)), (int)(b << 29));
+  const unsigned e = b & 0x7f800000u;
+  if (e == 0u || e == 0x7f800000u) r = (b << 1) == 0u ? 0.0 : (double)x;  // zero; denormal, Inf, NaN
+  return r;
+}
+
+// sum_k d_k added in order in FP64, of FP32 values.  GB300 issues an FP64 warp
+// instruction every 16 cycles an SM, so Q additions and conversions a cell
+// would cost several times the cell's HBM time.  When every partial sum is
+// representable the additions round nothing and their order does not matter,
+// so the sum is taken in 64-bit integers instead: with E the largest exponent
+// of the d_k, every nonzero d_k of exponent >= E - 24 is a multiple of
+// 2^(E-24-23) below 2^(E+1), and up to 32 of them add to less than 2^(E+6) =
+// 2^53 units.  Anything else (a wider spread, denormals, Inf or NaN) takes
+// the FP64 additions.  *finite: every d_k is finite.
+template <int Q>
+__device__ __forceinline__ double sum_in_order(const float (&d)[Q], bool* finite) {
+  static_assert(Q <= 32, "the integer sum holds 32 terms");
+  unsigned hi = 0u, lo = 0xffffffffu;  // largest and smallest nonzero magnitude (lo: minus one)
+#pragma unroll
+  for (int k = 0; k < Q; ++k) {
+    const unsigned mag = __float_as_uint(d[k]) & 0x7fffffffu;
+    hi = max(hi, mag);
+    lo = min(lo, mag - 1u);  // zero wraps to the largest value
+  }
+  const int E = (int)(hi >> 23);
+  *finite = E < 255;
+  if (hi == 0u) return 0.0;
+  lo += 1u;
+  // (E > 24: the window holds no denormals)
+  if (E < 255 && E > 24 && (int)(lo >> 23) >= E - 24) {
+    long long acc = 0;
+#pragma unroll
+    for (int k = 0; k < Q; ++k) {
+      const unsigned b = __float_as_uint(d[k]);
+      const int s = (int)b >> 31;
+      const int e = (int)((b >> 23) & 0xffu) - (E - 24);
+      const int m = (int)((b & 0x7fffffu) | 0x800000u);
+      // zero: exponent field 0, far below the window
+      const int w = e >= 0 ? 1 << e : 0;
+      acc += (long long)((m ^ s) - s) * (long long)w;
+    }
+    // acc times 2^(E - 127 - 47), of at most 53 significant bits, assembled
+    const unsigned long long u = acc < 0 ? 0ull - (unsigned long long)acc : (unsigned long long)acc;
+    if (u == 0ull) return 0.0;
+    const int lz = __clzll((long long)u);
+    const unsigned long long man = ((u << lz) >> 11) & 0xfffffffffffffull;
+    const unsigned long long bits = ((unsigned long long)(1023 + 63 - lz + E - 174) << 52) | man;
+    return __longlong_as_double((long long)(acc < 0 ? bits | 0x8000000000000000ull : bits));
+  }
+  double r = 0.0;
+#pragma unroll
+  for (int k = 0; k < Q; ++k) r = __dadd_rn(r, (double)d[k]);
+  return r;
+}
+template <int Q>
+__device__ __forceinline__ double sum_in_order(const double (&d)[Q], bool* finite) {
+  double r = 0.0;
+#pragma unroll
+  for (int k = 0; k < Q; ++k) r = __dadd_rn(r, d[k]);
+  *finite = isfinite(r);
+  return r;
+}
+
 // out[b * (NC + 3) + j]: j = 0 mass deviation, 1..NC solutes, NC+1 solid,
 // NC+2 count of non-finite cells (as a double).
+// Bound by the FP64 pipe (one warp instruction every 16 cycles an SM,
+// conversions included), so its work is kept off the cells that do not need
+// it: the populations add in integers (sum_in_order); a pure cell's h is
+// exactly the unit vector of its phase, whose zero terms add exactly nothing,
+// which leaves ceq + mu / (2 A) a solute and the sums over cells; elsewhere
+// only the phases present are evaluated.  256^3 cells, N = 4, K-1 = 2, a
+// quarter of them grains: 4.18 ms with every term in FP64, 0.67 ms so (the
+// state's planes alone take 0.25 ms to read; the FP64 pipe is 78 % busy).
 template <int Q, int NP, int NC, class Real, class Store>
-__global__ void __launch_bounds__(kRedThreads)
+__global__ void __launch_bounds__(kRedThreads, sizeof(Real) == 4 ? 4 : 2)
     invariants_kernel(const InvParams P, const Real* __restrict__ phi, const Real* __restrict__ mu,
                       const Store* __restrict__ f, double* __restrict__ partial) {
-  constexpr int NV = NC + 3;
-  double acc[NV];
+  constexpr int NV = NC + 3, NS = NP == 2 ? 1 : NP;
+  double acc[NC + 2];
 #pragma unroll
-  for (int j = 0; j < NV; ++j) acc[j] = 0.0;
-  const long long stride = (long long)gridDim.x * kRedThreads;
-  for (long long x = blockIdx.x * (long long)kRedThreads + threadIdx.x; x < P.cells; x += stride) {
-    const long long o = padded(x, P.nx, P.px);
-    double p[NP], m[NC];
-    if (NP == 2) {
-      p[1] = (double)phi[o];
-      p[0] = __dsub_rn(1.0, p[1]);
-    } else {
-#pragma unroll
-      for (int a = 0; a < NP; ++a) p[a] = (double)phi[a * P.plane + o];
+  for (int j = 0; j < NC + 2; ++j) acc[j] = 0.0;
+  int bad = 0;  // cells with a value that is not finite
+  // cell x = stride n + first: column and row advance with it (a grid holds
+  // fewer than 2^31 cells)
+  const unsigned stride = gridDim.x * kRedThreads, cells = (unsigned)P.cells, nx = (unsigned)P.nx;
+  const unsigned dcol = stride % nx, drow = stride / nx;
+  unsigned x = blockIdx.x * kRedThreads + threadIdx.x;
+  unsigned col = x % nx, row = x / nx;
+  for (; x < cells; x += stride) {
+    const long long o = col + (long long)P.px * row;
+    col += dcol;
+    row += drow;
+    if (col >= nx) {
+      col -= nx;
+      ++row;
     }
+    Real ps[NS], m[NC];
+    Real d[Q];
 #pragma unroll
-    for (int i = 0; i < NC; ++i) m[i] = (double)mu[i * P.plane + o];
-    double dm = 0.0;
+    for (int a = 0; a < NS; ++a) ps[a] = (phi + a * P.plane)[o];
 #pragma unroll
-    for (int k = 0; k < Q; ++k) dm = __dadd_rn(dm, (double)Codec<Store>::load(f[k * P.plane + o]));
-    double h[NP];
+    for (int i = 0; i < NC; ++i) m[i] = (mu + i * P.plane)[o];
 #pragma unroll
-    for (int a = 0; a < NP; ++a) h[a] = h_exact<NP>(p, a);
-    double v[NV];
-    v[0] = dm;
-    const double th = P.tdep ? __dadd_rn(P.theta_t, __dmul_rn(P.G, (double)(x / P.vlayer))) : 0.0;
+    for (int k = 0; k < Q; ++k) d[k] = Codec<Store>::load((f + k * P.plane)[o]);
+    bool finite;
+    const double dm = sum_in_order(d, &finite);
+    acc[0] = __dadd_rn(acc[0], dm);
+    bool fm = true;  // phi and mu finite
+#pragma unroll
+    for (int a = 0; a < NS; ++a) fm = fm && isfinite(ps[a]);
+#pragma unroll
+    for (int i = 0; i < NC; ++i) fm = fm && isfinite(m[i]);
+    bad += finite && fm ? 0 : 1;
+    const double th = P.tdep ? __dadd_rn(P.theta_t, __dmul_rn(P.G, (double)((long long)x / P.vlayer))) : 0.0;
+    double m64[NC], m0[NC];  // mu_i, and mu_i / (2 A) where every phase has the same A
 #pragma unroll
     for (int i = 0; i < NC; ++i) {
-      double c = 0.0;
+      m64[i] = widen(m[i]);
+      m0[i] = P.same_A ? __dmul_rn(m64[i], P.inv2A[0]) : 0.0;
+    }
+    // ceq_a,i(T) + mu_i / (2 A_a) of this lane's phase a
+    auto c_of = [&](int a, int i) {
+      double ce = P.ceq[0][i];
+#pragma unroll
+      for (int b = 1; b < NP; ++b)
+        if (a == b) ce = P.ceq[b][i];
+      if (P.tdep) {
+        double k = P.dceq_dT[0][i];
+#pragma unroll
+        for (int b = 1; b < NP; ++b)
+          if (a == b) k = P.dceq_dT[b][i];
+        ce = __dadd_rn(ce, __dmul_rn(k, th));
+      }
+      if (P.same_A) return __dadd_rn(ce, m0[i]);
+      double inv = P.inv2A[0];
+#pragma unroll
+      for (int b = 1; b < NP; ++b)
+        if (a == b) inv = P.inv2A[b];
+      return __dadd_rn(ce, __dmul_rn(m64[i], inv));
+    };
+    if (fm) {
+      // The phases present, in ascending order, in slots (the others at 0):
+      // a phase at 0 has h = 0 and adds 0 to every sum, exactly.
+      using Slot = typename std::conditional<NP == 2, double, Real>::type;  // (phi_0 of two phases: FP64)
+      Slot q[NP];
+      int id[NP], n = 0;
+#pragma unroll
+      for (int j = 0; j < NP; ++j) {
+        q[j] = Slot(0);
+        id[j] = 0;
+      }
 #pragma unroll
       for (int a = 0; a < NP; ++a) {
-        const double ce = P.tdep ? __dadd_rn(P.ceq[a][i], __dmul_rn(P.dceq_dT[a][i], th)) : P.ceq[a][i];
-        c = __dadd_rn(c, __dmul_rn(h[a], __dadd_rn(ce, __dmul_rn(m[i], P.inv2A[a]))));
+        Slot pa;
+        if (NP == 2)
+          pa = a == 0 ? (ps[0] == Real(0) ? Slot(1) : Slot(__dsub_rn(1.0, widen(ps[0])))) : Slot(widen(ps[0]));
+        else
+          pa = Slot(ps[NP == 2 ? 0 : a]);
+        if (pa == Slot(0)) continue;
+#pragma unroll
+        for (int j = 0; j <= a; ++j)
+          if (n == j) {
+            q[j] = pa;
+            id[j] = a;
+          }
+        ++n;
       }
-      v[1 + i] = c;
+      const bool pure = n == 1 && q[0] == Slot(1);
+      if (__all_sync(__activemask(), pure)) {  // h is the unit vector, exactly
+#pragma unroll
+        for (int i = 0; i < NC; ++i) acc[1 + i] = __dadd_rn(acc[1 + i], c_of(id[0], i));
+        if (id[0] > 0) acc[NC + 1] = __dadd_rn(acc[NC + 1], 1.0);
+      } else {
+        double c[NC], sol = 0.0;
+#pragma unroll
+        for (int i = 0; i < NC; ++i) c[i] = 0.0;
+#pragma unroll
+        for (int j = 0; j < NP; ++j) {
+          if (j >= n) break;
+          // h_exact; 2 p is exact, so 3 - 2 p is one rounding
+          const double qj = widen(q[j]);
+          double h = __dmul_rn(__dmul_rn(qj, qj), __fma_rn(-2.0, qj, 3.0));
+          if (n >= 3) {
+            double s = 0.0;
+#pragma unroll
+            for (int b = 0; b < NP; ++b)
+#pragma unroll
+              for (int g = b + 1; g < NP; ++g)
+                if (b != j && g != j && q[g] != Slot(0)) s = __dadd_rn(s, __dmul_rn(widen(q[b]), widen(q[g])));
+            h = __dadd_rn(h, __dmul_rn(__dmul_rn(2.0, qj), s));
+          }
+#pragma unroll
+          for (int i = 0; i < NC; ++i) {
+            const double t = __dmul_rn(h, c_of(id[j], i));
+            c[i] = j == 0 ? t : __dadd_rn(c[i], t);
+          }
+          if (id[j] > 0) sol = j == 0 ? h : __dadd_rn(sol, h);
+        }
+#pragma unroll
+        for (int i = 0; i < NC; ++i) acc[1 + i] = __dadd_rn(acc[1 + i], c[i]);
+        acc[NC + 1] = __dadd_rn(acc[NC + 1], sol);
+      }
+    } else {
+      double p[NP], c[NC], sol = 0.0;
+      if (NP == 2) {
+        p[1] = (double)ps[0];
+        p[0] = __dsub_rn(1.0, p[1]);
+      } else {
+#pragma unroll
+        for (int a = 0; a < NP; ++a) p[a] = (double)ps[NP == 2 ? 0 : a];
+      }
+#pragma unroll
+      for (int i = 0; i < NC; ++i) c[i] = 0.0;
+#pragma unroll
+      for (int a = 0; a < NP; ++a) {
+        const double h = h_exact<NP>(p, a);
+#pragma unroll
+        for (int i = 0; i < NC; ++i) c[i] = __dadd_rn(c[i], __dmul_rn(h, c_of(a, i)));
+        if (a > 0) sol = __dadd_rn(sol, h);
+      }
+#pragma unroll
+      for (int i = 0; i < NC; ++i) acc[1 + i] = __dadd_rn(acc[1 + i], c[i]);
+      acc[NC + 1] = __dadd_rn(acc[NC + 1], sol);
     }
-    double sol = 0.0;
-#pragma unroll
-    for (int a = 1; a < NP; ++a) sol = __dadd_rn(sol, h[a]);
-    v[NC + 1] = sol;
-    bool finite = isfinite(dm);
-#pragma unroll
-    for (int a = 0; a < NP; ++a) finite = finite && isfinite(p[a]);
-#pragma unroll
-    for (int i = 0; i < NC; ++i) finite = finite && isfinite(m[i]);
-    v[NC + 2] = finite ? 0.0 : 1.0;
-#pragma unroll
-    for (int j = 0; j < NV; ++j) acc[j] = __dadd_rn(acc[j], v[j]);
   }
   __shared__ double s_w[kRedThreads / 32][NV];
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
 #pragma unroll
   for (int j = 0; j < NV; ++j) {
-    const double w = warp_sum_butterfly(acc[j]);
+    const double w = warp_sum_butterfly(j < NC + 2 ? acc[j < NC + 2 ? j : 0] : (double)bad);
     if (lane == 0) s_w[warp][j] = w;
   }
   __syncthreads();
-  if (threadIdx.x == 0) {
-#pragma unroll
-    for (int j = 0; j < NV; ++j) {
-      double s = s_w[0][j];
-      for (int w = 1; w < kRedThreads / 32; ++w) s = __dadd_rn(s, s_w[w][j]);
-      partial[blockIdx.x * NV + j] = s;
-    }
+  if (threadIdx.x < NV) {
+    const int j = threadIdx.x;
+    double s = s_w[0][j];
+    for (int w = 1; w < kRedThreads / 32; ++w) s = __dadd_rn(s, s_w[w][j]);
+    partial[blockIdx.x * NV + j] = s;
   }
 }
 
-// Adds the block partials in block order (one thread).
+// Adds the block partials in block order, one thread a total: the chain of
+// `blocks` dependent FP64 additions is the time, so the partials are staged
+// in shared memory first, by every thread, a batch at a time.
+constexpr int kFinishThreads = 256;
 template <int NV>
-__global__ void invariants_finish_kernel(const double* __restrict__ partial, int blocks,
-                                         double* __restrict__ out) {
-  if (threadIdx.x != 0 || blockIdx.x != 0) return;
-  for (int j = 0; j < NV; ++j) {
-    double s = partial[j];
-    for (int b = 1; b < blocks; ++b) s = __dadd_rn(s, partial[b * NV + j]);
-    out[j] = s;
+__global__ void __launch_bounds__(kFinishThreads)
+    invariants_finish_kernel(const double* __restrict__ partial, int blocks, double* __restrict__ out) {
+  constexpr int kBatch = 512;
+  __shared__ double s_p[kBatch * NV];
+  double s = 0.0;
+  for (int b0 = 0; b0 < blocks; b0 += kBatch) {
+    const int n = min(kBatch, blocks - b0);
+    __syncthreads();
+    for (int i = threadIdx.x; i < n * NV; i += kFinishThreads) s_p[i] = partial[(long long)b0 * NV + i];
+    __syncthreads();
+    if (threadIdx.x < NV) {
+      int b = 0;
+      if (b0 == 0) s = s_p[b++ * NV + threadIdx.x];
+#pragma unroll 8
+      for (; b < n; ++b) s = __dadd_rn(s, s_p[b * NV + threadIdx.x]);
+    }
   }
+  if (threadIdx.x < NV) out[threadIdx.x] = s;
 }
 
 }  // namespace gpflbm

@@ -229,7 +229,7 @@ struct Impl {
     invariants_kernel<Q, NP, NC, Real, Store><<<blocks, kRedThreads, 0, s>>>(
         p, static_cast<const Real*>(phi), static_cast<const Real*>(mu),
         static_cast<const Store*>(f), partial);
-    invariants_finish_kernel<NC + 3><<<1, 32, 0, s>>>(partial, blocks, out);
+    invariants_finish_kernel<NC + 3><<<1, kFinishThreads, 0, s>>>(partial, blocks, out);
     return cudaGetLastError();
   }
 
