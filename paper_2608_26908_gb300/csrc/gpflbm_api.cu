@@ -774,7 +774,7 @@ gpflbm_status gpflbm_set_state(gpflbm_t h, const void* phi, const void* mu, cons
     e = cudaStreamWaitEvent(h->xfer, h->ev_mark, 0);
     if (e == cudaSuccess)
       e = h->ops->load_state(xparams(h), sp, sm, sf, own(h, h->lay.phi[to], rs), own(h, h->lay.mu[to], rs),
-                             own(h, h->lay.f[to], ss), clk + to, nullptr, (double)t0, h->xfer);
+                             own(h, h->lay.f[to], ss), clk + to, nullptr, (double)t0, !on_device, h->xfer);
     if (e == cudaSuccess) e = classify(h, to, h->xfer);
     if (e == cudaSuccess) e = cudaEventRecord(h->ev_loaded, h->xfer);
     if (e == cudaSuccess) e = cudaStreamWaitEvent(s, h->ev_loaded, 0);
@@ -794,7 +794,7 @@ gpflbm_status gpflbm_set_state(gpflbm_t h, const void* phi, const void* mu, cons
     if (e != cudaSuccess) return cuda_fail(h, e, "set_state: clock");
   } else {
     // device or pinned sources: every plane and the counters in one launch
-    e = h->ops->load_state(xparams(h), sp, sm, sf, phi_d, mu_d, f_d, clk, clk + 1, (double)t0, s);
+    e = h->ops->load_state(xparams(h), sp, sm, sf, phi_d, mu_d, f_d, clk, clk + 1, (double)t0, !on_device, s);
     if (e != cudaSuccess) return cuda_fail(h, e, "set_state: load");
   }
   e = classify(h, h->cur, s);
@@ -966,6 +966,7 @@ gpflbm_status gpflbm_get_fields(gpflbm_t h, unsigned field_mask, void* const* ds
   }
   cudaError_t e;
   if (any_direct) {
+    direct.link = !on_device;
     e = h->ops->fields(xparams(h), direct, s);
     if (e != cudaSuccess) return cuda_fail(h, e, "get_fields: kernel");
   }

@@ -37,6 +37,7 @@ struct FieldsIO {
   void* o_rho;
   void* o_u;
   void* o_dev;
+  bool link;  // a destination is host memory, written over the host link
 };
 
 struct Ops {
@@ -54,10 +55,10 @@ struct Ops {
   cudaError_t (*load)(const void* params, const void* src_phi, const void* src_mu,
                       const void* src_f, void* phi, void* mu, void* f, cudaStream_t s);
   // the whole state (src_f may be null) and the step counters (clock_b may
-  // be null), in one launch
+  // be null), in one launch; link: the sources are host memory
   cudaError_t (*load_state)(const void* params, const void* src_phi, const void* src_mu,
                             const void* src_f, void* phi, void* mu, void* f, double* clock_a,
-                            double* clock_b, double t0, cudaStream_t s);
+                            double* clock_b, double t0, bool link, cudaStream_t s);
   cudaError_t (*fields)(const void* params, const FieldsIO& io, cudaStream_t s);
   cudaError_t (*invariants)(const InvParams& p, const void* phi, const void* mu, const void* f,
                             double* partial, int blocks, double* out, cudaStream_t s);
@@ -65,11 +66,15 @@ struct Ops {
   cudaError_t (*classify)(const void* params, const void* phi, unsigned char* flags, cudaStream_t s);
 };
 
-// Grid of the exchange kernels (state load, field write-back): two CTAs of
-// 256 threads per SM in a grid-stride loop.  That keeps enough accesses in
-// flight for the host link and for HBM, and leaves room on every SM for the
-// other of the two, which may run at the same time on another stream.
-inline unsigned exchange_blocks(long long items, int threads) {
+// Grid of the exchange kernels (state load, field write-back): a grid-stride
+// loop over `per_sm` CTAs of 256 threads per SM.  Two keep enough accesses in
+// flight for the host link and leave room on every SM for the other of the
+// two kernels, which may run at the same time on another stream; between
+// device buffers nothing runs beside them, and HBM wants more loads in
+// flight (1001^2 cells, one a thread: the load 21.5 us with two, 14.0 us with
+// eight).
+constexpr int kLinkCtas = 2, kDeviceCtas = 8;
+inline unsigned exchange_blocks(long long items, int threads, int per_sm) {
   static int sms = 0;
   if (sms == 0) {
     int dev = 0, v = 0;
@@ -79,8 +84,8 @@ inline unsigned exchange_blocks(long long items, int threads) {
     else
       return (unsigned)((items + threads - 1) / threads);  // one item per thread
   }
-  const long long need = (items + threads - 1) / threads;
-  return (unsigned)(need < 2LL * sms ? need : 2LL * sms);
+  const long long need = (items + threads - 1) / threads, cap = (long long)per_sm * sms;
+  return (unsigned)(need < cap ? need : cap);
 }
 
 // QQ: lattice size (0 = D2Q9 in 2D, D3Q19 in 3D; 27 = D3Q27).
@@ -173,7 +178,7 @@ struct Impl {
 
   static cudaError_t load_state(const void* params, const void* src_phi, const void* src_mu,
                                 const void* src_f, void* phi, void* mu, void* f, double* clock_a,
-                                double* clock_b, double t0, cudaStream_t s) {
+                                double* clock_b, double t0, bool link, cudaStream_t s) {
     const DevParams<Real>& P = *static_cast<const DevParams<Real>*>(params);
     const long long cells = (long long)P.n[0] * P.n[1] * P.n[2];
     constexpr int V = 16 / (int)sizeof(Real);  // one 16-byte word of each source plane
@@ -181,7 +186,7 @@ struct Impl {
     const bool vec = P.n[0] % V == 0 && al16(src_phi) && al16(src_mu) && al16(src_f);
     const int threads = 256;
     const long long items = vec ? cells / V : cells;
-    const unsigned blocks = exchange_blocks(items, threads);
+    const unsigned blocks = exchange_blocks(items, threads, link ? kLinkCtas : kDeviceCtas);
     const Real* sp = static_cast<const Real*>(src_phi);
     const Real* sm = static_cast<const Real*>(src_mu);
     const Real* sf = static_cast<const Real*>(src_f);
@@ -199,13 +204,26 @@ struct Impl {
   static cudaError_t fields(const void* params, const FieldsIO& io, cudaStream_t s) {
     const DevParams<Real>& P = *static_cast<const DevParams<Real>*>(params);
     const long long cells = (long long)P.n[0] * P.n[1] * P.n[2];
+    constexpr int V = 16 / (int)sizeof(Real);  // one 16-byte word of each plane
+    auto al16 = [](const void* p) { return (reinterpret_cast<uintptr_t>(p) & 15u) == 0; };
     const int threads = 256;
-    const unsigned blocks = exchange_blocks(cells, threads);
-    fields_kernel<D, Q, NP, NC, Real, Store, Real><<<blocks, threads, 0, s>>>(
-        P, static_cast<const Real*>(io.phi), static_cast<const Real*>(io.mu),
-        static_cast<const Store*>(io.f), io.clock, static_cast<Real*>(io.o_phi),
-        static_cast<Real*>(io.o_mu), static_cast<Real*>(io.o_c), static_cast<Real*>(io.o_f),
-        static_cast<Real*>(io.o_rho), static_cast<Real*>(io.o_u), static_cast<Real*>(io.o_dev));
+    // A grid too small to give every SM a CTA of V cells a thread is bound by a
+    // thread's own chain, and takes one cell a thread (FP64 128^2: 7.5 us
+    // against 11.2 us with V = 2).
+    const bool vec = P.n[0] % V == 0 && cells / V >= 152 * threads && al16(io.o_phi) && al16(io.o_mu) && al16(io.o_c) &&
+                     al16(io.o_f) && al16(io.o_rho) && al16(io.o_u) && al16(io.o_dev);
+    const unsigned blocks = exchange_blocks(vec ? cells / V : cells, threads, io.link ? kLinkCtas : kDeviceCtas);
+    auto go = [&](auto kernel) {
+      kernel<<<blocks, threads, 0, s>>>(
+          P, static_cast<const Real*>(io.phi), static_cast<const Real*>(io.mu), static_cast<const Store*>(io.f),
+          io.clock, static_cast<Real*>(io.o_phi), static_cast<Real*>(io.o_mu), static_cast<Real*>(io.o_c),
+          static_cast<Real*>(io.o_f), static_cast<Real*>(io.o_rho), static_cast<Real*>(io.o_u),
+          static_cast<Real*>(io.o_dev));
+    };
+    if (vec)
+      go(fields_kernel<D, Q, NP, NC, Real, Store, Real, V>);
+    else
+      go(fields_kernel<D, Q, NP, NC, Real, Store, Real, 1>);
     return cudaGetLastError();
   }
 
