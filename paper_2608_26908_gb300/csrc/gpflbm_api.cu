@@ -288,6 +288,9 @@ void fill_params(gpflbm_t h, DevParams<Real>& P) {
   P.G = (Real)p.G;
   P.inv_tau_f = (Real)(1.0 / p.tau_f);
   P.force_pre = (Real)(1.0 - 0.5 / p.tau_f);
+  P.omega = Real(1) - P.inv_tau_f;
+  P.pre9 = Real(9) * P.force_pre;
+  P.pre3 = Real(-3) * P.force_pre;
   P.q_floor = (Real)p.q_floor;
   P.theta0 = -p.undercool - p.G * p.v0;
   P.GV = p.G * p.V;

@@ -168,6 +168,8 @@ struct DevParams {
   // k of a cell away from the edges lands.  Host-computed, so that each
   // access is one 64-bit add of a parameter to the cell's address.
   long long f_at[27], f_to[27];
+  // 1 - 1/tau_f, 9 (1 - 1/(2 tau_f)) and -3 (1 - 1/(2 tau_f)), in Real
+  Real omega, pre9, pre3;
 };
 
 // 1/x rounded to nearest: the same value as the IEEE division 1/x, by the
@@ -187,6 +189,31 @@ __device__ __forceinline__ float add_rn(float a, float b) { return __fadd_rn(a, 
 __device__ __forceinline__ double add_rn(double a, double b) { return __dadd_rn(a, b); }
 __device__ __forceinline__ float sub_rn(float a, float b) { return __fsub_rn(a, b); }
 __device__ __forceinline__ double sub_rn(double a, double b) { return __dsub_rn(a, b); }
+
+// Comparisons with 0 and 1 without the FP64 pipe (an FP64 comparison costs
+// as much as an FP64 addition): the same truth values, NaN included.
+__device__ __forceinline__ bool is_zero(float x) { return x == 0.0f; }
+__device__ __forceinline__ bool is_zero(double x) { return (__double_as_longlong(x) << 1) == 0; }
+__device__ __forceinline__ bool is_one(float x) { return x == 1.0f; }
+__device__ __forceinline__ bool is_one(double x) { return __double_as_longlong(x) == 0x3ff0000000000000ll; }
+__device__ __forceinline__ bool is_positive(float x) { return x > 0.0f; }
+__device__ __forceinline__ bool is_positive(double x) {
+  const long long b = __double_as_longlong(x);
+  return b > 0 && b <= 0x7ff0000000000000ll;
+}
+
+// 1/sqrt(x) (FP64: a square root and a division take three times the FP64
+// instructions).
+__device__ __forceinline__ float rsqrt_of(float x) { return 1.0f / sqrtf(x); }
+__device__ __forceinline__ double rsqrt_of(double x) { return rsqrt(x); }
+
+// (Real)v of v >= 0 without the FP64 pipe.
+__device__ __forceinline__ void real_of(int v, float& r) { r = (float)v; }
+__device__ __forceinline__ void real_of(int v, double& r) {
+  const int lz = __clz(v);
+  const unsigned m = (unsigned)v << (lz & 31);
+  r = v == 0 ? 0.0 : __hiloint2double((int)(((unsigned)(1023 + 31 - lz) << 20) | ((m >> 11) & 0xfffffu)), (int)(m << 21));
+}
 
 template <class Real>
 __device__ __forceinline__ int fold_axis(const DevParams<Real>& P, int i, int a) {
@@ -402,10 +429,10 @@ __device__ __forceinline__ void collide(const DevParams<Real>& P, const Real* dk
                                         const Real* u, const Real* F, Put&& put) {
   using Lat = Lattice<Q>;
   constexpr int D = Lat::D;
-  const Real itau = P.inv_tau_f, pre = P.force_pre, omega = Real(1) - itau;
+  const Real itau = P.inv_tau_f, pre = P.force_pre, omega = P.omega, pre9 = P.pre9;
   // every product and sum rounded as written (fma_rn etc.), so that the two
   // 3D kernels, which both collide liquid cells, give the same bits
-  const Real irho = mul_rn(itau, rho), pre9 = mul_rn(Real(9), pre);
+  const Real irho = mul_rn(itau, rho);
   Real uu = Real(0), uF = Real(0), v[D], z[D];
 #pragma unroll
   for (int a = 0; a < D; ++a) {
@@ -416,23 +443,28 @@ __device__ __forceinline__ void collide(const DevParams<Real>& P, const Real* dk
     z[a] = fma_rn(Real(4.5), ru, mul_rn(pre9, F[a]));
   }
   const Real alpha =
-      fma_rn(itau, fma_rn(mul_rn(Real(-1.5), rho), uu, drho), mul_rn(mul_rn(Real(-3), pre), uF));
+      fma_rn(itau, fma_rn(mul_rn(Real(-1.5), rho), uu, drho), mul_rn(P.pre3, uF));
   put(0, fma_rn(omega, dk[0], mul_rn(Real(Lat::w(0)), alpha)));
 #pragma unroll
   for (int k = 1; k < Q; ++k) {
     if (Lat::opp(k) < k) continue;  // each pair once, at its first index
     const int kb = Lat::opp(k);
-    Real cu = Real(0), cz = Real(0), cv = Real(0);
+    // (the first term is not added to a zero: the compiler keeps that addition)
+    Real cu, cz, cv;
+    bool first = true;
 #pragma unroll
     for (int a = 0; a < D; ++a) {
-      if (Lat::c(k, a) > 0) {
-        cu += u[a];
-        cz += z[a];
-        cv += v[a];
-      } else if (Lat::c(k, a) < 0) {
-        cu -= u[a];
-        cz -= z[a];
-        cv -= v[a];
+      const int c = Lat::c(k, a);
+      if (c == 0) continue;
+      if (first) {
+        cu = c > 0 ? u[a] : -u[a];
+        cz = c > 0 ? z[a] : -z[a];
+        cv = c > 0 ? v[a] : -v[a];
+        first = false;
+      } else {
+        cu = c > 0 ? cu + u[a] : cu - u[a];
+        cz = c > 0 ? cz + z[a] : cz - z[a];
+        cv = c > 0 ? cv + v[a] : cv - v[a];
       }
     }
     const Real wk = Real(Lat::w(k));

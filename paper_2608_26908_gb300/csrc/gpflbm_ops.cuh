@@ -88,6 +88,9 @@ inline unsigned exchange_blocks(long long items, int threads, int per_sm) {
   return (unsigned)(need < cap ? need : cap);
 }
 
+// FP64 2D grids of at most this many 32x8 tiles take the small tiles.
+constexpr unsigned kSmall2DBlocks = 304;
+
 // QQ: lattice size (0 = D2Q9 in 2D, D3Q19 in 3D; 27 = D3Q27).
 // EXT: the step kernels of the extended model -- turned crystal axes and
 // temperature-dependent equilibrium compositions (a separate table, so that
@@ -110,6 +113,8 @@ struct Impl {
       if (e == cudaSuccess)
         e = cudaFuncSetAttribute(step2d_kernel<NP, NC, Real, Store, true, EXT>,
                                  cudaFuncAttributeMaxDynamicSharedMemorySize, (int)SZ::bytes);
+      // (the small FP64 tiles fit the default limit)
+      static_assert(sizeof(Real) == 4 || Step2D<NP, NC, Real, Store, true>::bytes <= 48 * 1024, "small tile");
     } else {
       e = cudaFuncSetAttribute(step3d_kernel<NP, NC, Real, Store, false, Q, EXT>,
                                cudaFuncAttributeMaxDynamicSharedMemorySize, (int)step3d_bytes);
@@ -128,9 +133,25 @@ struct Impl {
   static cudaError_t step_fused(const void* params, const StepIO& io, cudaStream_t s) {
     const DevParams<Real>& P = *static_cast<const DevParams<Real>*>(params);
     if constexpr (D == 2) {
-      const dim3 grid((P.n[0] + SZ::OX - 1) / SZ::OX, (P.n[1] + SZ::OY - 1) / SZ::OY);
       const Step2DIO sio = {io.phi_in, io.phi_out, io.mu_in, io.mu_out,
                             io.f_in,   io.f_out,   io.clock_in, io.clock_out};
+      auto tiles = [&](auto z) {
+        using T = decltype(z);
+        return dim3((P.n[0] + T::OX - 1) / T::OX, (P.n[1] + T::OY - 1) / T::OY);
+      };
+      if constexpr (sizeof(Real) == 8) {
+        using SS = Step2D<NP, NC, Real, Store, true>;
+        const dim3 big = tiles(SZ());
+        if (big.x * big.y <= kSmall2DBlocks) {
+          const dim3 grid = tiles(SS());
+          if (P.shrink)
+            step2d_kernel<NP, NC, Real, Store, true, EXT, true><<<grid, SS::NT, SS::bytes, s>>>(P, sio);
+          else
+            step2d_kernel<NP, NC, Real, Store, false, EXT, true><<<grid, SS::NT, SS::bytes, s>>>(P, sio);
+          return cudaGetLastError();
+        }
+      }
+      const dim3 grid = tiles(SZ());
       if (P.shrink)
         step2d_kernel<NP, NC, Real, Store, true, EXT><<<grid, SZ::NT, SZ::bytes, s>>>(P, sio);
       else
