@@ -190,6 +190,10 @@ __device__ __forceinline__ double add_rn(double a, double b) { return __dadd_rn(
 __device__ __forceinline__ float sub_rn(float a, float b) { return __fsub_rn(a, b); }
 __device__ __forceinline__ double sub_rn(double a, double b) { return __dsub_rn(a, b); }
 
+// Programmatic dependent launch (no effect in a kernel launched without it).
+__device__ __forceinline__ void launch_dependents() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
+__device__ __forceinline__ void wait_for_previous() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+
 // Comparisons with 0 and 1 without the FP64 pipe (an FP64 comparison costs
 // as much as an FP64 addition): the same truth values, NaN included.
 __device__ __forceinline__ bool is_zero(float x) { return x == 0.0f; }

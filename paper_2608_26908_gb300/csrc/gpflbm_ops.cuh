@@ -88,6 +88,24 @@ inline unsigned exchange_blocks(long long items, int threads, int per_sm) {
   return (unsigned)(need < cap ? need : cap);
 }
 
+// Launches a kernel that waits for its predecessor in the stream by itself
+// (wait_for_previous): its CTAs may be placed while the predecessor's last ones
+// run, where that one allows it (launch_dependents).
+template <class... Par, class... Arg>
+cudaError_t launch_dependent(void (*kernel)(Par...), dim3 grid, int threads, size_t smem, cudaStream_t s, Arg&&... arg) {
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = grid;
+  cfg.blockDim = dim3(threads);
+  cfg.dynamicSmemBytes = smem;
+  cfg.stream = s;
+  cudaLaunchAttribute attr[1];
+  attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  attr[0].val.programmaticStreamSerializationAllowed = 1;
+  cfg.attrs = attr;
+  cfg.numAttrs = 1;
+  return cudaLaunchKernelEx(&cfg, kernel, Par(arg)...);
+}
+
 // FP64 2D grids of at most this many 32x8 tiles take the small tiles.
 constexpr unsigned kSmall2DBlocks = 304;
 
@@ -144,18 +162,15 @@ struct Impl {
         const dim3 big = tiles(SZ());
         if (big.x * big.y <= kSmall2DBlocks) {
           const dim3 grid = tiles(SS());
-          if (P.shrink)
-            step2d_kernel<NP, NC, Real, Store, true, EXT, true><<<grid, SS::NT, SS::bytes, s>>>(P, sio);
-          else
-            step2d_kernel<NP, NC, Real, Store, false, EXT, true><<<grid, SS::NT, SS::bytes, s>>>(P, sio);
-          return cudaGetLastError();
+          return launch_dependent(P.shrink ? step2d_kernel<NP, NC, Real, Store, true, EXT, true>
+                                           : step2d_kernel<NP, NC, Real, Store, false, EXT, true>,
+                                  grid, SS::NT, SS::bytes, s, P, sio);
         }
       }
       const dim3 grid = tiles(SZ());
-      if (P.shrink)
-        step2d_kernel<NP, NC, Real, Store, true, EXT><<<grid, SZ::NT, SZ::bytes, s>>>(P, sio);
-      else
-        step2d_kernel<NP, NC, Real, Store, false, EXT><<<grid, SZ::NT, SZ::bytes, s>>>(P, sio);
+      return launch_dependent(P.shrink ? step2d_kernel<NP, NC, Real, Store, true, EXT, false>
+                                       : step2d_kernel<NP, NC, Real, Store, false, EXT, false>,
+                              grid, SZ::NT, SZ::bytes, s, P, sio);
     } else {
       // the tiling (twice over in z when one launch takes both passes)
       const unsigned gz = (P.v_hi - P.v_lo + S3::ZS - 1) / S3::ZS;

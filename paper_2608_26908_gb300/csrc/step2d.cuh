@@ -126,6 +126,11 @@ __global__ void __launch_bounds__(Step2D<NP, NC, Real, Store, SMALL>::NT, Step2D
   const int fy = inner_tile ? gy : fold_axis(P, gy, 1);
   const int g = fy * px + fx;  // a plane holds fewer than 2^31 cells
   const int r2 = (ty + 1) * W2 + tx + 1;  // this cell in the R1-plus-ring layout
+  // Programmatic dependent launch: the next step's CTAs may be placed as this
+  // one's retire, and do what stands above; every read and write of the state
+  // comes after the wait, which returns once the step before has finished and
+  // its writes are visible.
+  wait_for_previous();
   const double t_now = io.clock_in[0];
   if (blockIdx.x == 0 && blockIdx.y == 0 && tid == 0) io.clock_out[0] = t_now + 1.0;
   const Real theta_base = Real(P.theta0) - Real(P.GV) * Real(t_now);
@@ -359,6 +364,7 @@ __global__ void __launch_bounds__(Step2D<NP, NC, Real, Store, SMALL>::NT, Step2D
     if (tx < BX - 1) face(0);
     if (ty < BY - 1) face(1);
     __syncthreads();
+    launch_dependents();
     if (!inner) return;
 #pragma unroll
     for (int sidx = 0; sidx < NS; ++sidx) (phi_out + sidx * P.plane)[g] = ph[NP == 2 ? 1 : sidx];
@@ -671,6 +677,7 @@ __global__ void __launch_bounds__(Step2D<NP, NC, Real, Store, SMALL>::NT, Step2D
   __syncthreads();
 
   // 3. inner cells: mu^{n+1}, phi^{n+1}, pulled f^{n+1}
+  launch_dependents();
   if (!inner) return;
 #pragma unroll
   for (int sidx = 0; sidx < NS; ++sidx) (phi_out + sidx * P.plane)[g] = out[NP == 2 ? 1 : sidx];
