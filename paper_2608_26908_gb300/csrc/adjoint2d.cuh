@@ -193,7 +193,7 @@ __global__ void __launch_bounds__(Adj2D<Real>::NT, Adj2D<Real>::MIN_CTAS) adj2d_
   const long long o = (long long)fy * P.px + fx;
   const int h2 = (ty + 1) * W2 + tx + 1;  // this cell in the tile + two-cell halo
   const bool inner = tx >= 1 && tx <= BX - 2 && ty >= 1 && ty <= BY - 2 && gx < nx && gy < ny;
-  const Real theta_base = Real(P.theta0) - Real(P.GV) * Real(io.clock[0]);
+  const Real theta_base = theta_at(P, io.clock[0]);
   const bool walls = (P.wall[0] | P.wall[1]) != 0;
   const Real e = P.inv2A[1] - P.inv2A[0];
   const Real mob = P.mob_eps * P.eps;  // 1 / tau_phi
@@ -368,7 +368,7 @@ __global__ void __launch_bounds__(Adj2D<Real>::NT, Adj2D<Real>::MIN_CTAS) adj2d_
     const Real c10 = (P.ceq[1][0] - P.ceq[0][0]) + (P.dceq_dT[1][0] - P.dceq_dT[0][0]) * th + mu0 * e;
     lmu -= Aown * e * (Hs(s1) - Hs(s0));
     lsp += -Aown * c10 * dHs(s1) - Aown * (mu1 - mu0) * e * dHs(s1);
-    lsp += Aown * Real(P.GV) * (P.dceq_dT[1][0] - P.dceq_dT[0][0]) * dHs(s1);
+    lsp += Aown * P.GV_r * (P.dceq_dT[1][0] - P.dceq_dT[0][0]) * dHs(s1);
     ls += Aown * c10 * dHs(s0);
   }
   bool multi = false;

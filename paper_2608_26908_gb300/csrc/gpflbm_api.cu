@@ -294,6 +294,8 @@ void fill_params(gpflbm_t h, DevParams<Real>& P) {
   P.q_floor = (Real)p.q_floor;
   P.theta0 = -p.undercool - p.G * p.v0;
   P.GV = p.G * p.V;
+  P.theta0_r = (Real)P.theta0;
+  P.GV_r = (Real)P.GV;
   P.v_lo = 0;
   P.v_hi = h->D == 3 ? h->grid.nz : h->grid.ny;
   P.zbase = 0;
@@ -354,6 +356,7 @@ void slab_views(gpflbm_t h, DevParams<Real>& P, DevParams<Real>& X) {
   X = P;
   X.n[2] = h->v_hi - h->v_lo;
   X.theta0 = P.theta0 + (double)P.G * h->v_lo;  // T at owned plane v is T at grid plane v_lo + v
+  X.theta0_r = (Real)X.theta0;
   X.v_lo = 0;
   X.v_hi = X.n[2];
   X.zbase = 0;

@@ -170,6 +170,7 @@ struct DevParams {
   long long f_at[27], f_to[27];
   // 1 - 1/tau_f, 9 (1 - 1/(2 tau_f)) and -3 (1 - 1/(2 tau_f)), in Real
   Real omega, pre9, pre3;
+  Real theta0_r, GV_r;  // theta0, GV
 };
 
 // 1/x rounded to nearest: the same value as the IEEE division 1/x, by the
@@ -206,6 +207,29 @@ __device__ __forceinline__ bool is_positive(double x) {
   return b > 0 && b <= 0x7ff0000000000000ll;
 }
 
+// (double)x by integer arithmetic: GB300 converts on its FP64 pipe, one warp
+// instruction every 16 cycles an SM.  (A zero of either sign gives +0.)
+__device__ __forceinline__ double widen(double x) { return x; }
+__device__ __forceinline__ double widen(float x) {
+  const unsigned b = __float_as_uint(x);
+  double r = __hiloint2double((int)((b & 0x80000000u) | (((b & 0x7fffffffu) >> 3) + 0x38000000u)), (int)(b << 29));
+  const unsigned e = b & 0x7f800000u;
+  if (e == 0u || e == 0x7f800000u) r = (b << 1) == 0u ? 0.0 : (double)x;  // zero; denormal, Inf, NaN
+  return r;
+}
+
+// (Real)x of an integer |x| < 2^63 by integer arithmetic, rounded to nearest
+// even, for the same reason: a CTA's warps would queue for the FP64 pipe
+// before their first instruction (eutectic2d 1024x512: 16.3 -> 15.9 us a step).
+__device__ __forceinline__ void narrow(double x, double& r) { r = x; }
+__device__ __forceinline__ void narrow(double x, float& r) {
+  const unsigned hi = (unsigned)__double2hiint(x), lo = (unsigned)__double2loint(x);
+  const unsigned rem = lo & 0x1fffffffu;
+  unsigned b = (hi & 0x80000000u) | ((((hi >> 20) & 0x7ffu) - 896u) << 23) | ((hi & 0xfffffu) << 3) | (lo >> 29);
+  b += rem > 0x10000000u || (rem == 0x10000000u && (b & 1u)) ? 1u : 0u;
+  r = hi << 1 == 0u ? 0.0f : __uint_as_float(b);  // |x| >= 1, or zero
+}
+
 // 1/sqrt(x) (FP64: a square root and a division take three times the FP64
 // instructions).
 __device__ __forceinline__ float rsqrt_of(float x) { return 1.0f / sqrtf(x); }
@@ -217,6 +241,14 @@ __device__ __forceinline__ void real_of(int v, double& r) {
   const int lz = __clz(v);
   const unsigned m = (unsigned)v << (lz & 31);
   r = v == 0 ? 0.0 : __hiloint2double((int)(((unsigned)(1023 + 31 - lz) << 20) | ((m >> 11) & 0xfffffu)), (int)(m << 21));
+}
+
+// theta = T - T_E at vertical index 0 and time t; theta + G v at index v.
+template <class Real>
+__device__ __forceinline__ Real theta_at(const DevParams<Real>& P, double t) {
+  Real tr;
+  narrow(t, tr);
+  return P.theta0_r - P.GV_r * tr;
 }
 
 template <class Real>
@@ -940,17 +972,6 @@ __device__ __forceinline__ double warp_sum_butterfly(double v) {
 #pragma unroll
   for (int off = 16; off > 0; off >>= 1) v = __dadd_rn(v, __shfl_xor_sync(0xffffffffu, v, off));
   return v;
-}
-
-// (double)x by integer arithmetic: GB300 converts on its FP64 pipe, one warp
-// instruction every 16 cycles an SM.  (A zero of either sign gives +0.)
-__device__ __forceinline__ double widen(double x) { return x; }
-__device__ __forceinline__ double widen(float x) {
-  const unsigned b = __float_as_uint(x);
-  double r = __hiloint2double((int)((b & 0x80000000u) | (((b & 0x7fffffffu) >> 3) + 0x38000000u)), (int)(b << 29));
-  const unsigned e = b & 0x7f800000u;
-  if (e == 0u || e == 0x7f800000u) r = (b << 1) == 0u ? 0.0 : (double)x;  // zero; denormal, Inf, NaN
-  return r;
 }
 
 // sum_k d_k added in order in FP64, of FP32 values.  GB300 issues an FP64 warp

@@ -133,7 +133,7 @@ __global__ void __launch_bounds__(Step2D<NP, NC, Real, Store, SMALL>::NT, Step2D
   wait_for_previous();
   const double t_now = io.clock_in[0];
   if (blockIdx.x == 0 && blockIdx.y == 0 && tid == 0) io.clock_out[0] = t_now + 1.0;
-  const Real theta_base = Real(P.theta0) - Real(P.GV) * Real(t_now);
+  const Real theta_base = theta_at(P, t_now);
   const bool obs = (P.wall[0] | P.wall[1]) != 0 && obstacle(P, fx, fy, 0);
   Real vf;
   real_of(fy, vf);
@@ -168,6 +168,14 @@ __global__ void __launch_bounds__(Step2D<NP, NC, Real, Store, SMALL>::NT, Step2D
   };
   auto PH = [&](int a, int i) -> Real { return plane_of(s_phi, C2, a, i); };   // phi^n
   auto PN = [&](int a, int i) -> Real { return plane_of(s_pn, NT, a, i); };    // phi^{n+1}
+  // every load of the cell is issued before the first value is looked at (the
+  // ring's test, in a branch of its own, would hold the loads after it back)
+  Store fk[Q];
+#pragma unroll
+  for (int k = 0; k < Q; ++k) fk[k] = at_bytes(f_in + g, P.f_at[k]);
+  Real mu[NC];
+#pragma unroll
+  for (int i = 0; i < NC; ++i) mu[i] = (mu_in + i * P.plane)[g];
   Real ph[NP];
   load_phases<NP>(phi_in, g, P.plane, ph);
   bool liquid = pure_liquid(ph) && !obs;  // the tile's cells, for the liquid-tile path
@@ -220,12 +228,8 @@ __global__ void __launch_bounds__(Step2D<NP, NC, Real, Store, SMALL>::NT, Step2D
       stage(rv, rr);
     }
   };
-  Real mu[NC];
 #pragma unroll
-  for (int i = 0; i < NC; ++i) {
-    mu[i] = (mu_in + i * P.plane)[g];
-    s_mu[i * NT + tid] = mu[i];
-  }
+  for (int i = 0; i < NC; ++i) s_mu[i * NT + tid] = mu[i];
   // moments, U, F (drag, buoyancy and, with SHRINK, the shrinkage force fs)
   // and the collision of this cell's populations into shared memory
   auto lbm_cell = [&](const Real* dk, Real fsx, Real fsy) {
@@ -292,7 +296,7 @@ __global__ void __launch_bounds__(Step2D<NP, NC, Real, Store, SMALL>::NT, Step2D
   {
     Real dk[Q];
 #pragma unroll
-    for (int k = 0; k < Q; ++k) dk[k] = Codec<Store>::load(at_bytes(f_in + g, P.f_at[k]));
+    for (int k = 0; k < Q; ++k) dk[k] = Codec<Store>::load(fk[k]);
     if constexpr (SHRINK) {
 #pragma unroll
       for (int k = 0; k < Q; ++k) s_fs[k * NT + tid] = Codec<Store>::put(dk[k]);  // exact round trip
@@ -375,7 +379,7 @@ __global__ void __launch_bounds__(Step2D<NP, NC, Real, Store, SMALL>::NT, Step2D
       Real src = Real(0);
       if constexpr (EXT) {
 #pragma unroll
-        for (int a = 0; a < NP; ++a) src -= Real(P.GV) * P.dceq_dT[a][i] * (a == 0 ? Real(1) : Real(0));
+        for (int a = 0; a < NP; ++a) src -= P.GV_r * P.dceq_dT[a][i] * (a == 0 ? Real(1) : Real(0));
       }
       (mu_out + i * P.plane)[g] = mu[i] + (-div - src) * P.chi_pure[0];
     }
@@ -709,7 +713,7 @@ __global__ void __launch_bounds__(Step2D<NP, NC, Real, Store, SMALL>::NT, Step2D
       const Real div = (Ji[tid] - Ji[tid - 1]) + (Ji[NT + tid] - Ji[NT + tid - BX]);
       Real src = ((ceq_of(1, i) - ceq_of(0, i)) + mu[i] * dinv) * dh;
       // -(dT/dt) sum_a (dc_a/dT)_mu h_a^{n+1}, dT/dt = -G V
-      if constexpr (EXT) src -= Real(P.GV) * (P.dceq_dT[0][i] + (P.dceq_dT[1][i] - P.dceq_dT[0][i]) * hn);
+      if constexpr (EXT) src -= P.GV_r * (P.dceq_dT[0][i] + (P.dceq_dT[1][i] - P.dceq_dT[0][i]) * hn);
       (mu_out + i * P.plane)[g] = mu[i] + (-div - src) * ichi;
     }
   } else {
@@ -733,7 +737,7 @@ __global__ void __launch_bounds__(Step2D<NP, NC, Real, Store, SMALL>::NT, Step2D
       if constexpr (EXT) {
         // -(dT/dt) sum_a (dc_a/dT)_mu h_a^{n+1}, dT/dt = -G V
 #pragma unroll
-        for (int a = 0; a < NP; ++a) src -= Real(P.GV) * P.dceq_dT[a][i] * hn[a];
+        for (int a = 0; a < NP; ++a) src -= P.GV_r * P.dceq_dT[a][i] * hn[a];
       }
       (mu_out + i * P.plane)[g] = mu[i] + (-div - src) * ichi;
     }

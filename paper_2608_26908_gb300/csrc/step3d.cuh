@@ -142,7 +142,7 @@ __device__ __forceinline__ void general_tile(const DevParams<Real>& P, const Ste
   const bool owner = tx >= 1 && tx <= BX - 2 && ty >= 1 && ty <= BY - 2 && gx < nx && gy < ny;
   const double t_now = io.clock_in[0];
   if (bx == 0 && by == 0 && bz == 0 && tid == 0) io.clock_out[0] = t_now + 1.0;
-  const Real theta_base = Real(P.theta0) - Real(P.GV) * Real(t_now);
+  const Real theta_base = theta_at(P, t_now);
   // EXT: ceq_a,i(T) at vertical index v, T - T_E = theta_base + G v
   auto ceq_of = [&](int a, int i, int v) -> Real {
     if constexpr (EXT)
@@ -761,7 +761,7 @@ __device__ __forceinline__ void general_tile(const DevParams<Real>& P, const Ste
           Real src = Real(0);
           if constexpr (EXT) {
 #pragma unroll
-            for (int a = 0; a < NP; ++a) src -= Real(P.GV) * P.dceq_dT[a][i] * (a == 0 ? Real(1) : Real(0));
+            for (int a = 0; a < NP; ++a) src -= P.GV_r * P.dceq_dT[a][i] * (a == 0 ? Real(1) : Real(0));
           }
           mu_out[i * P.plane + g] = liquid_mu(P, mu, div, src);
         }
@@ -807,7 +807,7 @@ __device__ __forceinline__ void general_tile(const DevParams<Real>& P, const Ste
           if constexpr (EXT) {
             // -(dT/dt) sum_a (dc_a/dT)_mu h_a^{n+1}, dT/dt = -G V
 #pragma unroll
-            for (int a = 0; a < NP; ++a) src -= Real(P.GV) * P.dceq_dT[a][i] * hn[a];
+            for (int a = 0; a < NP; ++a) src -= P.GV_r * P.dceq_dT[a][i] * hn[a];
           }
           mu_out[i * P.plane + g] = mu + (-div - src) * ichi;
         }

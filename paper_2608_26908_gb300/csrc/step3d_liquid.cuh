@@ -68,7 +68,7 @@ __device__ __forceinline__ void liquid_tile(const DevParams<Real>& P, const Step
   const bool owner = tx >= 1 && tx <= BX - 2 && ty >= 1 && ty <= BY - 2 && gx < nx && gy < ny;
   const double t_now = io.clock_in[0];
   if (bx == 0 && by == 0 && bz == 0 && tid == 0) io.clock_out[0] = t_now + 1.0;
-  const Real theta_base = Real(P.theta0) - Real(P.GV) * Real(t_now);
+  const Real theta_base = theta_at(P, t_now);
   auto ceq_of = [&](int a, int i, int v) -> Real {
     if constexpr (EXT)
       return fma_rn(P.dceq_dT[a][i], fma_rn(P.G, Real(v), theta_base), P.ceq[a][i]);
@@ -185,7 +185,7 @@ __device__ __forceinline__ void liquid_tile(const DevParams<Real>& P, const Step
         Real src = Real(0);
         if constexpr (EXT) {
 #pragma unroll
-          for (int a = 0; a < NP; ++a) src -= Real(P.GV) * P.dceq_dT[a][i] * (a == 0 ? Real(1) : Real(0));
+          for (int a = 0; a < NP; ++a) src -= P.GV_r * P.dceq_dT[a][i] * (a == 0 ? Real(1) : Real(0));
         }
         mu_out[i * P.plane + g] = liquid_mu(P, mu, div, src);
       }
