@@ -209,6 +209,7 @@ __global__ void __launch_bounds__(Adj2D<Real>::NT, Adj2D<Real>::MIN_CTAS) adj2d_
   // 0. per-cell values: own cell, then the outer ring
   const Real s0 = __ldg(io.s0 + o), s1 = __ldg(io.s1 + o), mu0 = __ldg(io.mu0 + o);
   const bool obs = walls && obstacle(P, fx, fy, 0);
+  bool liquid = is_zero(s0) && is_zero(s1) && !obs;
   Macro2<Real> m;
   Real Aown;
   {
@@ -247,6 +248,7 @@ __global__ void __launch_bounds__(Adj2D<Real>::NT, Adj2D<Real>::MIN_CTAS) adj2d_
     q = (long long)qy * P.px + qx;
     const Real rs0 = __ldg(io.s0 + q), rs1 = __ldg(io.s1 + q), rmu = __ldg(io.mu0 + q);
     robs = walls && obstacle(P, qx, qy, 0);
+    liquid = liquid && is_zero(rs0) && is_zero(rs1) && !robs;
     Real dk[9];
 #pragma unroll
     for (int k = 0; k < 9; ++k) dk[k] = __ldg(io.d0 + k * plane + q);
@@ -266,7 +268,11 @@ __global__ void __launch_bounds__(Adj2D<Real>::NT, Adj2D<Real>::MIN_CTAS) adj2d_
   Aown = obs ? Real(0) : io.lmu1[o] / (P.inv2A[0] + Hs(s1) * e);
   sc[S::AA * C2 + h2] = Aown;
   if (tid < S::RING) sc[S::AA * C2 + rc] = robs ? Real(0) : io.lmu1[q] / rden;
-  __syncthreads();
+  // Liquid tile: no solid in the tile and its halo before or after the step,
+  // and no obstacle.  The antitrapping and phase-field terms are then exactly
+  // zero, and what forms, stores and gathers them is left out (the other lines
+  // are the same, and the bits with them).
+  const bool lean = __syncthreads_and(liquid);
 
   // 1. solute faces, by their lower cell a (tile + two-cell halo coordinates)
   auto solute_face = [&](int ia, int ja, int d) {
@@ -313,7 +319,7 @@ __global__ void __launch_bounds__(Adj2D<Real>::NT, Adj2D<Real>::MIN_CTAS) adj2d_
       cf[S::F_SPA] -= L * Real(0.5) * ua * c0a * dHs(s1a);
       cf[S::F_SPB] -= L * Real(0.5) * ub * c0b * dHs(s1b);
       // antitrapping -a eps liq dc dphi n_d (liq, n at time n)
-      if (P.at_eps != Real(0)) {
+      if (!lean && P.at_eps != Real(0)) {
         const Real g_n = s0b - s0a;
         const Real g_t = Real(0.25) * (sc[S::S0 * C2 + ca + st] + sc[S::S0 * C2 + cb + st] -
                                        sc[S::S0 * C2 + ca - st] - sc[S::S0 * C2 + cb - st]);
@@ -345,7 +351,8 @@ __global__ void __launch_bounds__(Adj2D<Real>::NT, Adj2D<Real>::MIN_CTAS) adj2d_
       }
     }
 #pragma unroll
-    for (int v = 0; v < NF; ++v) sf[(d * NF + v) * C2 + ca] = cf[v];
+    for (int v = 0; v < NF; ++v)
+      if (v < S::F_SA || !lean) sf[(d * NF + v) * C2 + ca] = cf[v];
   };
   solute_face(tx + 1, ty + 1, 0);
   solute_face(tx + 1, ty + 1, 1);
@@ -372,7 +379,7 @@ __global__ void __launch_bounds__(Adj2D<Real>::NT, Adj2D<Real>::MIN_CTAS) adj2d_
     ls += Aown * c10 * dHs(s0);
   }
   bool multi = false;
-  if (!obs) {
+  if (!lean && !obs) {
     unsigned act = 0;
 #pragma unroll
     for (int dy = -1; dy <= 1; ++dy)
@@ -385,17 +392,19 @@ __global__ void __launch_bounds__(Adj2D<Real>::NT, Adj2D<Real>::MIN_CTAS) adj2d_
 
   if (inner) {
     lmu += F(0, S::F_MUA, h2) + F(1, S::F_MUA, h2) + F(0, S::F_MUB, h2 - 1) + F(1, S::F_MUB, h2 - W2);
-    ls += F(0, S::F_SA, h2) + F(1, S::F_SA, h2) + F(0, S::F_SB, h2 - 1) + F(1, S::F_SB, h2 - W2);
-    // antitrapping across x-faces (transverse y) and y-faces (transverse x)
-    ls += F(0, S::F_T, h2 - W2) + F(0, S::F_T, h2 - W2 - 1) - F(0, S::F_T, h2 + W2) - F(0, S::F_T, h2 + W2 - 1);
-    ls += F(1, S::F_T, h2 - 1) + F(1, S::F_T, h2 - 1 - W2) - F(1, S::F_T, h2 + 1) - F(1, S::F_T, h2 + 1 - W2);
-    if (P.bc[1] == kWall) {  // the wall mirrors a-t / a+t onto the row next to it
-      if (gy == 0) ls -= F(0, S::F_T, h2) + F(0, S::F_T, h2 - 1);
-      if (gy == ny - 1) ls += F(0, S::F_T, h2) + F(0, S::F_T, h2 - 1);
-    }
-    if (P.bc[0] == kWall) {
-      if (gx == 0) ls -= F(1, S::F_T, h2) + F(1, S::F_T, h2 - W2);
-      if (gx == nx - 1) ls += F(1, S::F_T, h2) + F(1, S::F_T, h2 - W2);
+    if (!lean) {
+      ls += F(0, S::F_SA, h2) + F(1, S::F_SA, h2) + F(0, S::F_SB, h2 - 1) + F(1, S::F_SB, h2 - W2);
+      // antitrapping across x-faces (transverse y) and y-faces (transverse x)
+      ls += F(0, S::F_T, h2 - W2) + F(0, S::F_T, h2 - W2 - 1) - F(0, S::F_T, h2 + W2) - F(0, S::F_T, h2 + W2 - 1);
+      ls += F(1, S::F_T, h2 - 1) + F(1, S::F_T, h2 - 1 - W2) - F(1, S::F_T, h2 + 1) - F(1, S::F_T, h2 + 1 - W2);
+      if (P.bc[1] == kWall) {  // the wall mirrors a-t / a+t onto the row next to it
+        if (gy == 0) ls -= F(0, S::F_T, h2) + F(0, S::F_T, h2 - 1);
+        if (gy == ny - 1) ls += F(0, S::F_T, h2) + F(0, S::F_T, h2 - 1);
+      }
+      if (P.bc[0] == kWall) {
+        if (gx == 0) ls -= F(1, S::F_T, h2) + F(1, S::F_T, h2 - W2);
+        if (gx == nx - 1) ls += F(1, S::F_T, h2) + F(1, S::F_T, h2 - W2);
+      }
     }
     Real gUx = F(0, S::F_UA, h2) + F(0, S::F_UB, h2 - 1);
     Real gUy = F(1, S::F_UA, h2) + F(1, S::F_UB, h2 - W2);
@@ -464,8 +473,9 @@ __global__ void __launch_bounds__(Adj2D<Real>::NT, Adj2D<Real>::MIN_CTAS) adj2d_
       io.ld0[k * plane + o] = omega * a[k] + gr + Real(Lat::c(k, 0)) * gmx + Real(Lat::c(k, 1)) * gmy;
     if (!obs) ls -= gphil;  // phil = 1 - s
     lmu += gB * P.gbeta_c[0] * P.inv2A[0];
-    io.gacc[2 * plane + o] +=
-        (double)(gB * (P.dcl_ref[0] + P.dceq_dT[0][0] * (theta_base + P.G * Real(fy)) + mu0 * P.inv2A[0]));
+    // (a zero adds exactly nothing: far from the solid most steps have none)
+    const Real gb = gB * (P.dcl_ref[0] + P.dceq_dT[0][0] * (theta_base + P.G * Real(fy)) + mu0 * P.inv2A[0]);
+    if (!is_zero(gb)) io.gacc[2 * plane + o] += widen(gb);
 
     // phase field: s' = clamp(u) where both phases are present, s' = s elsewhere
     if (multi) {
@@ -477,13 +487,15 @@ __global__ void __launch_bounds__(Adj2D<Real>::NT, Adj2D<Real>::MIN_CTAS) adj2d_
         const Real cob = P.obst * P.gamma[0][1] / P.eps;  // 16 gamma / (pi^2 eps^2)
         ls += lu * (Real(1) + Real(0.5) * mob * (Real(2) * cob - (Real(6) / P.eps) * (Real(1) - Real(2) * s0) * dpsi));
         lmu += lu * Real(0.5) * mob * (-(Real(6) / P.eps) * s0 * (Real(1) - s0) * dpsi_dmu);
-        io.gacc[0 * plane + o] += (double)(lu * (s1 - s0) / mob);
+        io.gacc[0 * plane + o] += widen(lu * (s1 - s0) / mob);
       }
     } else {
       ls += lsp;
     }
     io.lmu0[o] = lmu;
+    if (lean) io.ls0[o] = ls;
   }
+  if (lean) return;  // no phase-field faces
   __syncthreads();
 
   // 3. phase-field faces: lambda_V = (mob/2) gamma (lu(a) - lu(b)) through
@@ -516,7 +528,7 @@ __global__ void __launch_bounds__(Adj2D<Real>::NT, Adj2D<Real>::MIN_CTAS) adj2d_
           }
           cn = lV * dV[0];
           ct = Real(0.25) * lV * dV[1];
-          if (inner) io.gacc[1 * plane + o] += (double)(lV * dV[2]);
+          if (inner) io.gacc[1 * plane + o] += widen(lV * dV[2]);
         }
       }
       spf[(d * 2 + 0) * NT + tid] = cn;
