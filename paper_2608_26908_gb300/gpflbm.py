@@ -350,6 +350,20 @@ class Sim:
                                                          ctypes.byref(n)), "adjoint_workspace_bytes")
         return n.value
 
+    def _adjoint_workspace(self, horizon, ckpt_every):
+        """A workspace from torch's caching allocator, used on the current
+        stream, or None (the library allocates its own): a cudaMalloc and a
+        cudaFree of gigabytes in every call take as long as 40 adjoint steps of
+        512 x 512 cells."""
+        torch = self.torch
+        n = ctypes.c_size_t()
+        if lib().gpflbm_adjoint_workspace_bytes(self.h, int(horizon), int(ckpt_every), ctypes.byref(n)) != OK:
+            return None
+        try:
+            return torch.empty(n.value, dtype=torch.uint8, device="cuda")
+        except torch.cuda.OutOfMemoryError:
+            return None
+
     def adjoint(self, obj, horizon, ckpt_every, device=False, workspace=None):
         """Run `horizon` steps from the current state and the adjoint back.
 
@@ -357,7 +371,7 @@ class Sim:
         gbeta_c[0]) as a numpy array, dmu0 = dJ/dmu of the starting state (one
         plane; a device tensor if device=True).  The state is left at
         t0 + horizon.  workspace: optional uint8 device tensor of at least
-        adjoint_workspace_bytes() bytes (else the library allocates one).
+        adjoint_workspace_bytes() bytes (else one from torch's allocator).
         """
         torch = self.torch
         o = objective_struct(obj)
@@ -369,6 +383,8 @@ class Sim:
         else:
             dmu = np.empty(self.cells, dtype=self.dtype)
             dptr = ctypes.c_void_p(dmu.ctypes.data)
+        if workspace is None:
+            workspace = self._adjoint_workspace(horizon, ckpt_every)
         if workspace is not None:
             wptr, wbytes = ctypes.c_void_p(workspace.data_ptr()), workspace.numel()
         else:
