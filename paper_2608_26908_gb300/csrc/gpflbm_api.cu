@@ -98,9 +98,12 @@ gpflbm_status cuda_fail(gpflbm_t h, cudaError_t e, const char* where) {
 }
 
 // The kernel table the time steps use: the extended model's when a pair of
-// the problem's phases has a nonzero tilt or an equilibrium composition
-// depends on temperature.
-const Ops* stepper(gpflbm_t h) { return h->pf.tilted || h->pf.tdep ? h->ops_ext : h->ops; }
+// the problem's phases has a nonzero tilt, an equilibrium composition depends
+// on temperature, or, in 3D with three or four phases, the gradient energy is
+// anisotropic (the plain kernels leave that out there, see general_tile).
+const Ops* stepper(gpflbm_t h) {
+  return h->pf.tilted || h->pf.tdep || (h->D == 3 && h->NP > 2 && (h->pf.aniso || h->pd.aniso)) ? h->ops_ext : h->ops;
+}
 
 // Record the caller's stream's progress for asynchronous loads, once per
 // run of read-only calls (see gpflbm_s::ev_mark).
@@ -379,11 +382,25 @@ bool liquid_dispatch(gpflbm_t h) {
   return true;
 }
 
+// Segments a CTA of the liquid path marches: kLiquidGroup, fewer where that
+// would leave too few CTAs to fill the chip several times over.
+constexpr long long kLiquidCtas = 2000;
+int liquid_group(gpflbm_t h) {
+  using B = gpflbm::Block3D<float>;
+  const gpflbm_grid& g = h->grid;
+  const long long xy = (long long)((g.nx + B::BX - 3) / (B::BX - 2)) * ((g.ny + B::BY - 3) / (B::BY - 2));
+  const long long segs = (h->v_hi - h->v_lo + B::ZS - 1) / B::ZS;
+  int n = h->ops->store_size == 2 ? gpflbm::kLiquidGroup<__half> : 1;
+  while (n > 1 && xy * ((segs + n - 1) / n) < kLiquidCtas) --n;
+  return n;
+}
+
 void set_device_params(gpflbm_t h) {
   fill_params(h, h->pd);
   fill_params(h, h->pf);
   const int liq = liquid_dispatch(h) ? 1 : 0;
   h->pd.liq_dispatch = h->pf.liq_dispatch = liq;
+  h->pd.liq_group = h->pf.liq_group = liquid_group(h);
   slab_views(h, h->pd, h->xd);
   slab_views(h, h->pf, h->xf);
   h->inv.cells = h->cells;
@@ -697,8 +714,10 @@ gpflbm_status gpflbm_set_params(gpflbm_t h, const gpflbm_params* params) {
   drop_graphs(h);  // parameters are baked into captured launches
   ++h->mut;
   if (h->has_state && h->pf.liq_dispatch && !had) {
-    // the flags were not kept while every tile took the general path
+    // the flags were not kept while every tile took the general path (the
+    // liquid path also reads those of the buffer it writes)
     cudaError_t e = classify(h, h->cur, nullptr);
+    if (e == cudaSuccess) e = classify(h, 1 - h->cur, nullptr);
     if (e == cudaSuccess) e = cudaStreamSynchronize(nullptr);
     if (e != cudaSuccess) return cuda_fail(h, e, "set_params: liquid tiles");
   }

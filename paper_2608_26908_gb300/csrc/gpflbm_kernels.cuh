@@ -171,6 +171,7 @@ struct DevParams {
   // 1 - 1/tau_f, 9 (1 - 1/(2 tau_f)) and -3 (1 - 1/(2 tau_f)), in Real
   Real omega, pre9, pre3;
   Real theta0_r, GV_r;  // theta0, GV
+  int liq_group;        // 3D: segments a CTA of the liquid path takes
 };
 
 // 1/x rounded to nearest: the same value as the IEEE division 1/x, by the
@@ -326,29 +327,31 @@ __device__ __forceinline__ long long liquid_flag_index(int bx, int by, int v, in
 // where a wall mirrors the tile's own cells) on planes z0 - 2 .. z0 + ZS + 1
 // (folded like the cells) -- is flagged pure liquid.  Every thread of the CTA
 // calls it; the answer is uniform.
+// The flag of tile t (0 .. 8) of the 3 x 3 around (bx, by) in plane v (any
+// plane the reach names; set where the tile lies beyond a wall).
+template <class Real>
+__device__ __forceinline__ bool liquid_flag_near(const DevParams<Real>& P, const unsigned char* __restrict__ flags,
+                                                 int bx, int by, int v, int t, int gx, int gy) {
+  int c[2] = {bx + t % 3 - 1, by + t / 3 - 1};
+  const int n[2] = {gx, gy};
+  bool skip = false;
+#pragma unroll
+  for (int a = 0; a < 2; ++a) {
+    if (c[a] < 0 || c[a] >= n[a]) {
+      if (P.bc[a] == kWall) skip = true;
+      c[a] = c[a] < 0 ? c[a] + n[a] : c[a] - n[a];
+    }
+  }
+  return skip || flags[liquid_flag_index(c[0], c[1], fold_axis(P, v, 2), gx, gy)] != 0;
+}
+
 template <int ZS, class Real>
 __device__ __forceinline__ bool liquid_reach(const DevParams<Real>& P, const unsigned char* __restrict__ flags,
                                              int bx, int by, int z0, int gx, int gy) {
-  __shared__ int s_all;
-  if (threadIdx.x == 0) s_all = 1;
-  __syncthreads();
-  if (threadIdx.x < 9 * (ZS + 4)) {
-    const int t = threadIdx.x % 9;
-    const int v = fold_axis(P, z0 - 2 + (int)threadIdx.x / 9, 2);
-    int c[2] = {bx + t % 3 - 1, by + t / 3 - 1};
-    const int n[2] = {gx, gy};
-    bool skip = false;
-#pragma unroll
-    for (int a = 0; a < 2; ++a) {
-      if (c[a] < 0 || c[a] >= n[a]) {
-        if (P.bc[a] == kWall) skip = true;
-        c[a] = c[a] < 0 ? c[a] + n[a] : c[a] - n[a];
-      }
-    }
-    if (!skip && !flags[liquid_flag_index(c[0], c[1], v, gx, gy)]) s_all = 0;
-  }
-  __syncthreads();
-  return s_all != 0;
+  bool liquid = true;
+  if (threadIdx.x < 9 * (ZS + 4))
+    liquid = liquid_flag_near(P, flags, bx, by, z0 - 2 + (int)threadIdx.x / 9, threadIdx.x % 9, gx, gy);
+  return __syncthreads_and(liquid);
 }
 
 // ------------------------------------------------------------------ shared cell arithmetic
@@ -385,13 +388,18 @@ __device__ __forceinline__ void force_velocity(const DevParams<Real>& P, Real rh
   }
 }
 
-// Solute flux between two pure-liquid cells a, b (M = M0, h_l = 1):
-// J = -M0 (mu_b - mu_a) + (u_a c_a + u_b c_b) / 2, c = ceq_l + mu / (2 A_l).
+// Half the advective solute current of a pure-liquid cell along one axis:
+// u c / 2, c = ceq_l + mu / (2 A_l).
 template <class Real>
-__device__ __forceinline__ Real liquid_flux(const DevParams<Real>& P, Real ma, Real mb, Real ua, Real ub,
-                                            Real ceqa, Real ceqb) {
-  const Real adv = mul_rn(Real(0.5), fma_rn(ua, fma_rn(ma, P.inv2A[0], ceqa), mul_rn(ub, fma_rn(mb, P.inv2A[0], ceqb))));
-  return fma_rn(-P.M0, sub_rn(mb, ma), adv);
+__device__ __forceinline__ Real liquid_adv(const DevParams<Real>& P, Real u, Real mu, Real ceq) {
+  return mul_rn(u, mul_rn(Real(0.5), fma_rn(mu, P.inv2A[0], ceq)));
+}
+
+// Solute flux between two pure-liquid cells a, b (M = M0, h_l = 1), w their
+// halved currents: J = -M0 (mu_b - mu_a) + w_a + w_b.
+template <class Real>
+__device__ __forceinline__ Real liquid_flux(const DevParams<Real>& P, Real ma, Real mb, Real wa, Real wb) {
+  return fma_rn(-P.M0, sub_rn(mb, ma), add_rn(wa, wb));
 }
 
 // mu^{n+1} of an unchanged pure-liquid cell: mu + (-div - src) / (2 A_l)^-1.
@@ -432,6 +440,30 @@ __device__ __forceinline__ Real interp_dh(const Real* p, int b, int a) {
   return Real(2) * p[b] * s;
 }
 
+// drv_a = sum_b psi_b dh_b/dphi_a: with w_b = psi_b phi_b and T = sum phi,
+//   psi_a (6 phi_a (1 - phi_a) + 2 E_a) + 2 sum_{b != a} w_b (T - phi_a - phi_b),
+// E_a = sum_{b<g; b,g != a} phi_b phi_g (a fifth of the operations of
+// interp_dh pair by pair).
+template <int NP, class Real>
+__device__ __forceinline__ void driving_force(const Real* p, const Real* psi, Real* drv) {
+  Real w[NP], T = Real(0), W = Real(0), X = Real(0), e2 = Real(0);
+#pragma unroll
+  for (int b = 0; b < NP; ++b) {
+    w[b] = psi[b] * p[b];
+    e2 += T * p[b];
+    T += p[b];
+    W += w[b];
+    X += w[b] * p[b];
+  }
+#pragma unroll
+  for (int a = 0; a < NP; ++a) {
+    const Real t = T - p[a];  // the other phases
+    const Real cross = t * (W - w[a]) - (X - w[a] * p[a]);
+    const Real E = e2 - p[a] * t;
+    drv[a] = psi[a] * (Real(6) * p[a] * (Real(1) - p[a]) + Real(2) * E) + Real(2) * cross;
+  }
+}
+
 // dA/dq_j for A(q) = ac(q)^2 |q|^2, ac = 1 - delta (3 - 4 sum q^4 / |q|^4).
 // Only component j is returned, but it depends on all of q.
 template <int D, class Real>
@@ -460,7 +492,8 @@ __device__ __forceinline__ Real dAdq(const Real* q, Real delta, Real q_floor, in
 // equilibrium over tau plus the discrete force, collected by powers of c_k.
 // Opposite directions share alpha and the quadratic term and flip the linear
 // one, so each pair costs one evaluation.  put(k, value) stores a result.
-template <int Q, class Real, class Put>
+// ZFORCE: the force is along the last axis alone (F[a] = 0 before it).
+template <int Q, bool ZFORCE = false, class Real, class Put>
 __device__ __forceinline__ void collide(const DevParams<Real>& P, const Real* dk, Real drho, Real rho,
                                         const Real* u, const Real* F, Put&& put) {
   using Lat = Lattice<Q>;
@@ -472,11 +505,16 @@ __device__ __forceinline__ void collide(const DevParams<Real>& P, const Real* dk
   Real uu = Real(0), uF = Real(0), v[D], z[D];
 #pragma unroll
   for (int a = 0; a < D; ++a) {
-    uu = fma_rn(u[a], u[a], uu);
-    uF = fma_rn(u[a], F[a], uF);
+    uu = a == 0 ? mul_rn(u[a], u[a]) : fma_rn(u[a], u[a], uu);
     const Real ru = mul_rn(irho, u[a]);
-    v[a] = mul_rn(Real(3), fma_rn(pre, F[a], ru));
-    z[a] = fma_rn(Real(4.5), ru, mul_rn(pre9, F[a]));
+    if (ZFORCE && a < D - 1) {
+      v[a] = mul_rn(Real(3), ru);
+      z[a] = mul_rn(Real(4.5), ru);
+    } else {
+      uF = a == 0 || ZFORCE ? mul_rn(u[a], F[a]) : fma_rn(u[a], F[a], uF);
+      v[a] = mul_rn(Real(3), fma_rn(pre, F[a], ru));
+      z[a] = fma_rn(Real(4.5), ru, mul_rn(pre9, F[a]));
+    }
   }
   const Real alpha =
       fma_rn(itau, fma_rn(mul_rn(Real(-1.5), rho), uu, drho), mul_rn(P.pre3, uF));
@@ -605,6 +643,36 @@ __device__ __forceinline__ void project_simplex(Real* u, int m) {
 #pragma unroll
   for (int j = 0; j < NMAX; ++j)
     if (j < m) u[j] = u[j] - theta > Real(0) ? u[j] - theta : Real(0);
+}
+
+// The same for the phases whose bit of act is set (two or more), the others
+// to 0; u in place.
+template <int NP, class Real>
+__device__ __forceinline__ void project_present(Real* u, unsigned act) {
+  Real s[NP];
+#pragma unroll
+  for (int j = 0; j < NP; ++j) s[j] = act & (1u << j) ? u[j] : Real(-1e30);
+#pragma unroll
+  for (int i = 0; i < NP; ++i)
+#pragma unroll
+    for (int j = 0; j + 1 < NP - i; ++j) {
+      const Real hi = s[j] < s[j + 1] ? s[j + 1] : s[j], lo = s[j] < s[j + 1] ? s[j] : s[j + 1];
+      s[j] = hi;
+      s[j + 1] = lo;
+    }
+  // (the absent phases sort last, and none of them passes the test)
+  Real run = s[0], tau = s[0] - Real(1);
+#pragma unroll
+  for (int j = 1; j < NP; ++j) {
+    run += s[j];
+    const Real t = (run - Real(1)) * Real(1.0 / (j + 1));
+    if (s[j] - t > Real(0)) tau = t;
+  }
+#pragma unroll
+  for (int j = 0; j < NP; ++j) {
+    const Real v = u[j] - tau;
+    u[j] = (act & (1u << j)) && v > Real(0) ? v : Real(0);
+  }
 }
 
 // ------------------------------------------------------------------ phase field

@@ -175,9 +175,9 @@ struct Impl {
       // the tiling (twice over in z when one launch takes both passes)
       const unsigned gz = (P.v_hi - P.v_lo + S3::ZS - 1) / S3::ZS;
       const dim3 grid((P.n[0] + S3::OX - 1) / S3::OX, (P.n[1] + S3::OY - 1) / S3::OY,
-                      S3::ONE_LAUNCH && P.liq_dispatch ? 2 * gz : gz);
+                      S3::ONE_LAUNCH && P.liq_dispatch ? gz + (gz + P.liq_group - 1) / P.liq_group : gz);
       const Step3DIO sio = {io.phi_in, io.phi_out, io.mu_in,    io.mu_out,    io.f_in,
-                            io.f_out,  io.clock_in, io.clock_out, io.flags_in, io.flags_out};
+                      io.f_out,  io.clock_in, io.clock_out, io.flags_in, io.flags_out};
       if (P.shrink)
         step3d_kernel<NP, NC, Real, Store, true, Q, EXT><<<grid, S3::NT, step3d_bytes, s>>>(P, sio);
       else
@@ -185,7 +185,8 @@ struct Impl {
       // the tiles whose reach is pure liquid (step3d_kernel returned there)
       if constexpr (!S3::ONE_LAUNCH) {
         if (P.liq_dispatch)
-          step3d_liquid_kernel<NP, NC, Real, Store, Q, EXT><<<grid, SL::NT, SL::bytes, s>>>(P, sio);
+          step3d_liquid_kernel<NP, NC, Real, Store, Q, EXT>
+              <<<dim3(grid.x, grid.y, (gz + P.liq_group - 1) / P.liq_group), SL::NT, SL::bytes, s>>>(P, sio);
       }
     }
     return cudaGetLastError();

@@ -34,14 +34,8 @@ namespace gpflbm {
 // is deep, and no general tile, whose lone march sets the step's tail,
 // runs long.
 template <class Real>
-struct Block3D;
-template <>
-struct Block3D<float> {
-  static constexpr int BX = 32, BY = 16, ZS = 6;
-};
-template <>
-struct Block3D<double> {
-  static constexpr int BX = 32, BY = 8, ZS = 16;
+struct Block3D {
+  static constexpr int BX = 32, BY = 16, ZS = sizeof(Real) == 4 ? 6 : 16;
 };
 
 template <int NP, int NC, class Real, class Store, int QQ = 19>
@@ -49,6 +43,9 @@ struct Step3D {
   static constexpr int BX = Block3D<Real>::BX, BY = Block3D<Real>::BY, ZS = Block3D<Real>::ZS;
   static constexpr int NT = BX * BY, Q = QQ;  // D3Q19 or D3Q27
   static constexpr int NS = PhiStore<NP>::NS;
+  // values of a phase-field face: two phases need the difference of their two
+  // fluxes alone (see pf_face)
+  static constexpr int NF = NP == 2 ? 1 : NP;
   // resident CTAs per SM the register budget is cut for: two (64 registers)
   // on D3Q19 in FP32, for any number of phases (three and four phases spill
   // a few dozen bytes, yet two CTAs of 64 registers beat one of 128: 1.79
@@ -71,14 +68,14 @@ struct Step3D {
   // phi^{n+1} of planes C and M (written in C, read by the solute faces
   // and the update of the next iteration); U_x, U_y of the same two planes
   // (U_z only enters this column's own z-face: registers)
-  static constexpr size_t pn = al(mask + 3 * C2);                   // 2 planes x NP x NT
-  static constexpr size_t u = al(pn + sizeof(Real) * 2 * NP * NT);   // 2 planes x 2 x NT
+  static constexpr size_t pn = al(mask + 3 * C2);                   // 2 planes x NS x NT
+  static constexpr size_t u = al(pn + sizeof(Real) * 2 * NS * NT);   // 2 planes x 2 x NT
   static constexpr size_t mu = al(u + sizeof(Real) * 2 * 2 * NT);    // 2 planes x NC x NT
   static constexpr size_t hl = al(mu + sizeof(Real) * 2 * NC * NT);  // 2 planes x NT
   static constexpr size_t chg = al(hl + sizeof(Real) * 2 * NT);      // 2 planes x NT bytes
   static constexpr size_t flux = al(chg + 2 * NT);                   // PF or solute in-plane faces
   static constexpr size_t flux_n =
-      NP * (PFX + PFY) > 2 * NC * NT ? NP * (PFX + PFY) : 2 * NC * NT;
+      NF * (PFX + PFY) > 2 * NC * NT ? NF * (PFX + PFY) : 2 * NC * NT;
   static constexpr size_t bytes = al(flux + sizeof(Real) * flux_n);
 };
 
@@ -140,6 +137,9 @@ __device__ __forceinline__ void general_tile(const DevParams<Real>& P, const Ste
   const int r2 = (ty + 1) * W2 + tx + 1;
   // inner columns of the tile write the tile's cells
   const bool owner = tx >= 1 && tx <= BX - 2 && ty >= 1 && ty <= BY - 2 && gx < nx && gy < ny;
+  // a wall at this column's +x, +y face
+  const bool shut_x = P.bc[0] == kWall && (gx + 1 == 0 || gx + 1 == nx);
+  const bool shut_y = P.bc[1] == kWall && (gy + 1 == 0 || gy + 1 == ny);
   const double t_now = io.clock_in[0];
   if (bx == 0 && by == 0 && bz == 0 && tid == 0) io.clock_out[0] = t_now + 1.0;
   const Real theta_base = theta_at(P, t_now);
@@ -150,6 +150,11 @@ __device__ __forceinline__ void general_tile(const DevParams<Real>& P, const Ste
     else
       return P.ceq[a][i];
   };
+  // Three and four phases: the plain kernels are for isotropic problems, and an
+  // anisotropic one takes the extended model's (the launcher's choice): with
+  // the anisotropic stencils in it the code outgrows the instruction cache
+  // (ncu: 4.0 of 14 stall cycles an issue wait for instructions, 0.4 without).
+  const bool aniso = (NP == 2 || EXT) && P.aniso != 0;
   const bool has_walls = (P.wall[0] | P.wall[1] | P.wall[2]) != 0;  // obstacle rows
   // vertical index of a plane the kernel reads: folded on the whole grid
   // (walls mirror, periodic wraps), then kept inside the planes the buffers
@@ -221,70 +226,101 @@ __device__ __forceinline__ void general_tile(const DevParams<Real>& P, const Ste
   unsigned xy_m1 = 0, xy_0 = 0;
 
   // phase-field z-face fluxes of this column: (C-1, C) carried, (C, C+1) new
-  Real pfz_lo[NP], pfz_hi[NP];
+  Real pfz_lo[S::NF], pfz_hi[S::NF];
   // solute z-face fluxes of this column: (M-1, M) carried, (M, M+1) new
   Real mz_lo[NC], mz_hi[NC];
   // U_z of this column in planes M and C
   Real uz_M = Real(0), uz_C = Real(0);
 #pragma unroll
-  for (int a = 0; a < NP; ++a) pfz_lo[a] = pfz_hi[a] = Real(0);
+  for (int a = 0; a < S::NF; ++a) pfz_lo[a] = pfz_hi[a] = Real(0);
 #pragma unroll
   for (int i = 0; i < NC; ++i) mz_lo[i] = mz_hi[i] = Real(0);
 
-  // face flux of the phase field between cells A and B (R1-plus-ring indices
-  // in planes pa, pb); normal axis d; t1, t2 the transverse steps (in-plane
-  // index offsets or plane offsets); returns the d-th component of
-  // -sum_{b != a} gamma_ab phi_b dA/dq(q_ab) for every phase
-  auto pf_flux = [&](int pa, int ia, int pb, int ib, int d, bool closed, Real* fl) {
+  // phi^{n+1} of plane p (slots of two)
+  auto PN = [&](int p, int a, int i) -> Real {
+    const Real* b = s_pn + slot2(p) * NS * NT;
+    if (NP == 2) return a == 0 ? Real(1) - b[i] : b[i];
+    return b[a * NT + i];
+  };
+
+  // Face flux of the phase field between cell A (plane pa, R1-plus-ring index
+  // ia) and its neighbour B along axis d: the d-th component of -sum_{b != a}
+  // gamma_ab phi_b dA/dq(q_ab) for every phase.  Two phases: q_01 = grad phi_1
+  // on the face (phi_0 + phi_1 = 1) and the update needs gamma dA/dq, the
+  // difference of the two fluxes, alone: V = dA/dq.  d is a run-time value so
+  // that the code is there once: with a copy a face the general path waits for
+  // its instructions (ncu: 2.4 of 14 stall cycles an issue).
+  constexpr int NF = S::NF;
+  auto pf_face = [&](int pa, int ia, int d, bool closed, Real* fl) {
 #pragma unroll
-    for (int a = 0; a < NP; ++a) fl[a] = Real(0);
-    // the cells the stencil reads
-    unsigned grp;
-    Real pf[NP], g3[NP][3];
-    if (d == 2) {
-      grp = MK(pa, ia) | MK(pb, ib) | MK(pa, ia + 1) | MK(pb, ib + 1) | MK(pa, ia - 1) |
-            MK(pb, ib - 1) | MK(pa, ia + W2) | MK(pb, ib + W2) | MK(pa, ia - W2) | MK(pb, ib - W2);
-    } else {
-      const int st = d == 0 ? W2 : 1;
-      grp = MK(pa, ia) | MK(pb, ib) | MK(pa, ia + st) | MK(pb, ib + st) | MK(pa, ia - st) |
-            MK(pb, ib - st) | MK(pa - 1, ia) | MK(pb - 1, ib) | MK(pa + 1, ia) | MK(pb + 1, ib);
+    for (int a = 0; a < NF; ++a) fl[a] = Real(0);
+    const int pb = d == 2 ? pa + 1 : pa, ib = ia + (d == 0 ? 1 : (d == 1 ? W2 : 0));
+    const int st = d == 0 ? W2 : 1;  // the first transverse step, in the plane
+    unsigned grp = MK(pa, ia) | MK(pb, ib);
+    // dA/dq = 2 q without anisotropy: only q_d, of the two cells, enters
+    if (aniso) {
+      grp |= MK(pa, ia + st) | MK(pb, ib + st) | MK(pa, ia - st) | MK(pb, ib - st);
+      if (d == 2)
+        grp |= MK(pa, ia + W2) | MK(pb, ib + W2) | MK(pa, ia - W2) | MK(pb, ib - W2);
+      else
+        grp |= MK(pa - 1, ia) | MK(pa - 1, ib) | MK(pa + 1, ia) | MK(pa + 1, ib);
     }
     if (__popc(grp) < 2 || closed) return;
-    // A phase whose mask bit is clear in every cell the stencil reads is
-    // exactly 0 there: its face value and gradient are 0, so every pair it
-    // belongs to has q = 0 and contributes exactly 0.  Such phases and pairs
-    // are skipped (two or three of the four phases at most interfaces).
-#pragma unroll
-    for (int a = 0; a < NP; ++a) {
-      pf[a] = Real(0);
-      g3[a][0] = g3[a][1] = g3[a][2] = Real(0);
-      if (!(grp & (1u << a))) continue;
-      const Real va = PH(pa, a, ia), vb = PH(pb, a, ib);
-      pf[a] = Real(0.5) * (va + vb);
-      g3[a][d] = vb - va;
-      if (!P.aniso) continue;  // dA/dq = 2 q: only q_d enters the flux
-      if (d == 2) {
-        g3[a][0] = Real(0.25) * (PH(pa, a, ia + 1) + PH(pb, a, ib + 1) - PH(pa, a, ia - 1) - PH(pb, a, ib - 1));
-        g3[a][1] = Real(0.25) * (PH(pa, a, ia + W2) + PH(pb, a, ib + W2) - PH(pa, a, ia - W2) - PH(pb, a, ib - W2));
-      } else {
-        const int st = d == 0 ? W2 : 1;  // the other in-plane axis
-        g3[a][1 - d] = Real(0.25) * (PH(pa, a, ia + st) + PH(pb, a, ib + st) - PH(pa, a, ia - st) - PH(pb, a, ib - st));
-        g3[a][2] = Real(0.25) * (PH(pa + 1, a, ia) + PH(pb + 1, a, ib) - PH(pa - 1, a, ia) - PH(pb - 1, a, ib));
-      }
+    auto at = [&](int p, int i) { return slot4(p) * NS * C2 + i; };
+    const int A = at(pa, ia), B = at(pb, ib);
+    // cells beside A and B along the second transverse axis
+    int ap = A, am = A, bp = B, bm = B;
+    if (aniso) {
+      ap = d == 2 ? A + W2 : at(pa + 1, ia);
+      am = d == 2 ? A - W2 : at(pa - 1, ia);
+      bp = d == 2 ? B + W2 : at(pa + 1, ib);
+      bm = d == 2 ? B - W2 : at(pa - 1, ib);
     }
-#pragma unroll
-    for (int a = 0; a < NP; ++a)
-#pragma unroll
-      for (int b = a + 1; b < NP; ++b) {
-        const Real gab = P.gamma[a][b];
-        if (gab == Real(0) || (grp & ((1u << a) | (1u << b))) != ((1u << a) | (1u << b))) continue;
-        Real q[3];
-#pragma unroll
-        for (int t = 0; t < 3; ++t) q[t] = pf[a] * g3[b][t] - pf[b] * g3[a][t];
-        const Real v = dAdq_pair<3, EXT>(P, a, b, q, d);
-        fl[a] -= gab * pf[b] * v;
-        fl[b] += gab * pf[a] * v;
+    // q from its components along d, along st and along the second transverse axis
+    auto flux = [&](int a, int b, Real qn, Real q1, Real q2) -> Real {
+      if (!aniso) return Real(2) * qn;
+      if constexpr (EXT) {  // the crystal axes may be turned: true axes
+        const Real q[3] = {d == 0 ? qn : q1, d == 1 ? qn : (d == 0 ? q1 : q2), d == 2 ? qn : q2};
+        Real v[3];
+        dAdq_vec_pair<3, true>(P, a, b, q, v);
+        return d == 0 ? v[0] : (d == 1 ? v[1] : v[2]);
+      } else {
+        const Real q[3] = {qn, q1, q2};
+        return dAdq<3>(q, P.delta[a][b], P.q_floor, 0);
       }
+    };
+    if constexpr (NP == 2) {
+      const Real* f = s_phi;
+      const Real g1 = aniso ? Real(0.25) * (f[A + st] + f[B + st] - f[A - st] - f[B - st]) : Real(0);
+      const Real g2 = aniso ? Real(0.25) * (f[ap] + f[bp] - f[am] - f[bm]) : Real(0);
+      fl[0] = flux(0, 1, f[B] - f[A], g1, g2);
+    } else {
+      // A phase whose mask bit is clear in every cell the stencil reads is
+      // exactly 0 there, and every pair it belongs to contributes exactly 0.
+      Real pf[NP], gn[NP], g1[NP], g2[NP];
+#pragma unroll
+      for (int a = 0; a < NP; ++a) {
+        const Real* f = s_phi + a * C2;
+        const Real va = f[A], vb = f[B];
+        pf[a] = Real(0.5) * (va + vb);
+        gn[a] = vb - va;
+        g1[a] = g2[a] = Real(0);
+        if (aniso) {
+          g1[a] = Real(0.25) * (f[A + st] + f[B + st] - f[A - st] - f[B - st]);
+          g2[a] = Real(0.25) * (f[ap] + f[bp] - f[am] - f[bm]);
+        }
+      }
+#pragma unroll
+      for (int a = 0; a < NP; ++a)
+#pragma unroll
+        for (int b = a + 1; b < NP; ++b) {
+          if ((grp & ((1u << a) | (1u << b))) != ((1u << a) | (1u << b))) continue;
+          const Real gv = P.gamma[a][b] * flux(a, b, pf[a] * gn[b] - pf[b] * gn[a], pf[a] * g1[b] - pf[b] * g1[a],
+                                               pf[a] * g2[b] - pf[b] * g2[a]);
+          fl[a] -= pf[b] * gv;
+          fl[b] += pf[a] * gv;
+        }
+    }
   };
 
   const int L0 = z0 - 2, L1 = z0 + ZS + 1;
@@ -368,15 +404,15 @@ __device__ __forceinline__ void general_tile(const DevParams<Real>& P, const Ste
             at_bytes(fo, P.f_to[k]) = Codec<Store>::put(val);
           });
         } else {
-        // push to x + c_k (periodic axes wrap; across a wall the population
-        // returns reversed into the cell)
-        const PushAxis X = push_axis(gx, nx, P.bc[0] == kWall, 1);
-        const PushAxis Y = push_axis(gy, ny, P.bc[1] == kWall, px);
-        const PushAxis Z = push_axis(C, nz, P.bc[2] == kWall, zst);
-        collide<Q>(P, dk, drho, rho, u, F, [&](int k, Real val) {
-          if (hdir != 0 && Lat::c(k, 2) != hdir) return;
-          push_store<Lat>(f_out, P.plane, gi, k, Codec<Store>::put(val), X, Y, Z);
-        });
+          // push to x + c_k (periodic axes wrap; across a wall the population
+          // returns reversed into the cell)
+          const PushAxis X = push_axis(gx, nx, P.bc[0] == kWall, 1);
+          const PushAxis Y = push_axis(gy, ny, P.bc[1] == kWall, px);
+          const PushAxis Z = push_axis(C, nz, P.bc[2] == kWall, zst);
+          collide<Q>(P, dk, drho, rho, u, F, [&](int k, Real val) {
+            if (hdir != 0 && Lat::c(k, 2) != hdir) return;
+            push_store<Lat>(f_out, P.plane, gi, k, Codec<Store>::put(val), X, Y, Z);
+          });
         }
       }
       }  // !SHRINK
@@ -417,79 +453,136 @@ __device__ __forceinline__ void general_tile(const DevParams<Real>& P, const Ste
     // without another barrier)
     if ((liq_hist & 7u) == 7u || !__syncthreads_or(pfC && mixed)) {
 #pragma unroll
-      for (int a = 0; a < NP; ++a) pfz_hi[a] = Real(0);
+      for (int a = 0; a < NF; ++a) pfz_hi[a] = Real(0);
     } else {
       if (pfC) {
-        // in-plane faces of plane C into shared memory
-        Real fl[NP];
-        const bool cx_hi = P.bc[0] == kWall && (gx + 1 == 0 || gx + 1 == nx);
-        pf_flux(C, r2, C, r2 + 1, 0, cx_hi, fl);
+        // f = 0: the first face of every row and column, by the lanes of two
+        // warps; 1, 2: the +x and +y faces into shared memory; 3: the z-face
+        // (C, C+1); 4, on the first plane: (C-1, C)
+        const int nf = C == z0 - 1 ? 5 : 4;
 #pragma unroll
-        for (int a = 0; a < NP; ++a) s_flux[a * (S::PFX + S::PFY) + ty * (BX + 1) + tx + 1] = fl[a];
-        if (tx == 0) {
-          const bool cx_lo = P.bc[0] == kWall && (gx == 0 || gx == nx);
-          pf_flux(C, r2 - 1, C, r2, 0, cx_lo, fl);
+        for (int f = 0; f < 5; ++f) {
+          if (f >= nf) continue;
+          int p = C, ia = r2, d = f == 0 ? 0 : min(f, 3) - 1, slot = 0;
+          bool closed = shut_x;
+          if (f == 0) {
+            const int e = tid - 32;
+            if (e < 0 || e >= BX + BY) continue;
+            if (e < BY) {
+              ia = (e + 1) * W2;
+              closed = P.bc[0] == kWall && (x0 == 1 || x0 - 1 == nx);
+              slot = e * (BX + 1);
+            } else {
+              d = 1;
+              ia = e - BY + 1;
+              closed = P.bc[1] == kWall && (y0 == 1 || y0 - 1 == ny);
+              slot = S::PFX + e - BY;
+            }
+          } else if (f == 1) {
+            slot = ty * (BX + 1) + tx + 1;
+          } else if (f == 2) {
+            closed = shut_y;
+            slot = S::PFX + (ty + 1) * BX + tx;
+          } else {
+            p = f == 3 ? C : C - 1;
+            closed = P.bc[2] == kWall && (p + 1 == 0 || p + 1 == nz);
+          }
+          Real fl[NF];
+          pf_face(p, ia, d, closed, fl);
+          if (f < 3) {
 #pragma unroll
-          for (int a = 0; a < NP; ++a) s_flux[a * (S::PFX + S::PFY) + ty * (BX + 1)] = fl[a];
-        }
-        const bool cy_hi = P.bc[1] == kWall && (gy + 1 == 0 || gy + 1 == ny);
-        pf_flux(C, r2, C, r2 + W2, 1, cy_hi, fl);
+            for (int a = 0; a < NF; ++a) s_flux[a * (S::PFX + S::PFY) + slot] = fl[a];
+          } else {
 #pragma unroll
-        for (int a = 0; a < NP; ++a) s_flux[a * (S::PFX + S::PFY) + S::PFX + (ty + 1) * BX + tx] = fl[a];
-        if (ty == 0) {
-          const bool cy_lo = P.bc[1] == kWall && (gy == 0 || gy == ny);
-          pf_flux(C, r2 - W2, C, r2, 1, cy_lo, fl);
-#pragma unroll
-          for (int a = 0; a < NP; ++a) s_flux[a * (S::PFX + S::PFY) + S::PFX + tx] = fl[a];
-        }
-        // z-faces of this column: (C, C+1), and (C-1, C) on the first plane
-        const bool cz_hi = P.bc[2] == kWall && (C + 1 == 0 || C + 1 == nz);
-        pf_flux(C, r2, C + 1, r2, 2, cz_hi, pfz_hi);
-        if (C == z0 - 1) {
-          const bool cz_lo = P.bc[2] == kWall && (C == 0 || C == nz);
-          pf_flux(C - 1, r2, C, r2, 2, cz_lo, pfz_lo);
+            for (int a = 0; a < NF; ++a) {
+              if (f == 3)
+                pfz_hi[a] = fl[a];
+              else
+                pfz_lo[a] = fl[a];
+            }
+          }
         }
       }
       __syncthreads();
       if (pfC && multi) {
-        Real div[NP], gc[NP][3];
-#pragma unroll
-        for (int a = 0; a < NP; ++a) {
-          const Real* fa = s_flux + a * (S::PFX + S::PFY);
-          div[a] = (fa[ty * (BX + 1) + tx + 1] - fa[ty * (BX + 1) + tx]) +
-                   (fa[S::PFX + (ty + 1) * BX + tx] - fa[S::PFX + ty * BX + tx]) + (pfz_hi[a] - pfz_lo[a]);
-          // a phase absent from the 3x3x3 neighbourhood has a zero central
-          // gradient, and its pairs contribute exactly 0 below
-          gc[a][0] = gc[a][1] = gc[a][2] = Real(0);
-          if (!(act & (1u << a))) continue;
-          gc[a][0] = Real(0.5) * (PH(C, a, r2 + 1) - PH(C, a, r2 - 1));
-          gc[a][1] = Real(0.5) * (PH(C, a, r2 + W2) - PH(C, a, r2 - W2));
-          gc[a][2] = Real(0.5) * (PH(C + 1, a, r2) - PH(C - 1, a, r2));
-        }
-        Real ph[NP];
-#pragma unroll
-        for (int a = 0; a < NP; ++a) ph[a] = out[a];
-        Real dadphi[NP];
-#pragma unroll
-        for (int a = 0; a < NP; ++a) dadphi[a] = Real(0);
-#pragma unroll
-        for (int a = 0; a < NP; ++a)
-#pragma unroll
-          for (int b = a + 1; b < NP; ++b) {
-            const Real gab = P.gamma[a][b];
-            if (gab == Real(0) || (act & ((1u << a) | (1u << b))) != ((1u << a) | (1u << b))) continue;
-            Real q[3], v[3];
-#pragma unroll
-            for (int t = 0; t < 3; ++t) q[t] = ph[a] * gc[b][t] - ph[b] * gc[a][t];
-            dAdq_vec_pair<3, EXT>(P, a, b, q, v);
-            dadphi[a] += gab * (v[0] * gc[b][0] + v[1] * gc[b][1] + v[2] * gc[b][2]);
-            dadphi[b] -= gab * (v[0] * gc[a][0] + v[1] * gc[a][1] + v[2] * gc[a][2]);
-          }
         const int fzC = vz(C);
         const Real theta = theta_base + P.G * Real(fzC);
         Real mu[NC];
 #pragma unroll
         for (int i = 0; i < NC; ++i) mu[i] = s_mu[(slot2(C) * NC + i) * NT + tid];
+        if constexpr (NP == 2) {
+          // Lambda is the mean of the two rates, so phi_1 moves by half their
+          // difference; the centre terms da/dphi are equal and cancel, and
+          // dh_1/dphi_1 = dh_0/dphi_0 = 6 s (1 - s)
+          const Real sv = out[1], s0 = out[0];
+          const Real div = (s_flux[ty * (BX + 1) + tx + 1] - s_flux[ty * (BX + 1) + tx]) +
+                           (s_flux[S::PFX + (ty + 1) * BX + tx] - s_flux[S::PFX + ty * BX + tx]) +
+                           (pfz_hi[0] - pfz_lo[0]);
+          Real dpsi = (P.S[1] - P.S[0]) * theta;
+#pragma unroll
+          for (int i = 0; i < NC; ++i)
+            dpsi -= mu[i] * (mu[i] * (P.inv4A[1] - P.inv4A[0]) + (ceq_of(1, i, fzC) - ceq_of(0, i, fzC)));
+          const Real rate = P.eps * P.gamma[0][1] * div - P.obst * (P.gamma[1][0] * s0 - P.gamma[0][1] * sv) -
+                            Real(6) * sv * s0 * dpsi;
+          Real v = sv + Real(0.5) * P.mob_eps * rate;
+          v = v < Real(0) ? Real(0) : (v > Real(1) ? Real(1) : v);
+          out[1] = v;
+          out[0] = Real(1) - v;
+        } else {
+        Real ph[NP];
+#pragma unroll
+        for (int a = 0; a < NP; ++a) ph[a] = out[a];
+        // central differences of phase a along axis t
+        auto grad = [&](int a, int t) -> Real {
+          return t == 0 ? Real(0.5) * (PH(C, a, r2 + 1) - PH(C, a, r2 - 1))
+                        : (t == 1 ? Real(0.5) * (PH(C, a, r2 + W2) - PH(C, a, r2 - W2))
+                                  : Real(0.5) * (PH(C + 1, a, r2) - PH(C - 1, a, r2)));
+        };
+        // the gradient energy's centre terms
+        Real dadphi[NP];
+#pragma unroll
+        for (int a = 0; a < NP; ++a) dadphi[a] = Real(0);
+        if (!aniso) {
+          // dA/dq = 2 q, q_ab = phi_a g_b - phi_b g_a: by the products g_a . g_b
+          Real G[NP][NP];
+#pragma unroll
+          for (int t = 0; t < 3; ++t) {
+            Real g[NP];
+#pragma unroll
+            for (int a = 0; a < NP; ++a) g[a] = grad(a, t);
+#pragma unroll
+            for (int a = 0; a < NP; ++a)
+#pragma unroll
+              for (int b = a; b < NP; ++b) G[a][b] = t == 0 ? g[a] * g[b] : G[a][b] + g[a] * g[b];
+          }
+#pragma unroll
+          for (int a = 0; a < NP; ++a)
+#pragma unroll
+            for (int b = a + 1; b < NP; ++b) {
+              const Real g2 = Real(2) * P.gamma[a][b];
+              dadphi[a] += g2 * (ph[a] * G[b][b] - ph[b] * G[a][b]);
+              dadphi[b] += g2 * (ph[b] * G[a][a] - ph[a] * G[a][b]);
+            }
+        } else {
+          Real gc[NP][3];
+#pragma unroll
+          for (int a = 0; a < NP; ++a)
+#pragma unroll
+            for (int t = 0; t < 3; ++t) gc[a][t] = grad(a, t);
+#pragma unroll
+          for (int a = 0; a < NP; ++a)
+#pragma unroll
+            for (int b = a + 1; b < NP; ++b) {
+              const Real gab = P.gamma[a][b];
+              if (gab == Real(0) || (act & ((1u << a) | (1u << b))) != ((1u << a) | (1u << b))) continue;
+              Real q[3], v[3];
+#pragma unroll
+              for (int t = 0; t < 3; ++t) q[t] = ph[a] * gc[b][t] - ph[b] * gc[a][t];
+              dAdq_vec_pair<3, EXT>(P, a, b, q, v);
+              dadphi[a] += gab * (v[0] * gc[b][0] + v[1] * gc[b][1] + v[2] * gc[b][2]);
+              dadphi[b] -= gab * (v[0] * gc[a][0] + v[1] * gc[a][1] + v[2] * gc[a][2]);
+            }
+        }
         Real psi[NP];
 #pragma unroll
         for (int b = 0; b < NP; ++b) {
@@ -498,41 +591,29 @@ __device__ __forceinline__ void general_tile(const DevParams<Real>& P, const Ste
           for (int i = 0; i < NC; ++i) sv -= mu[i] * mu[i] * P.inv4A[b] + mu[i] * ceq_of(b, i, fzC);
           psi[b] = sv;
         }
-        Real rate[NP];
+        Real drv[NP];
+        driving_force<NP>(ph, psi, drv);
+        Real rate[NP], lam = Real(0);
+        int na = 0;
 #pragma unroll
         for (int a = 0; a < NP; ++a) {
-          Real obst = Real(0), drv = Real(0);
+          Real obst = Real(0);
 #pragma unroll
-          for (int b = 0; b < NP; ++b) {
+          for (int b = 0; b < NP; ++b)
             if (b != a) obst += P.gamma[a][b] * ph[b];
-            drv += psi[b] * interp_dh<NP>(ph, b, a);
-          }
-          rate[a] = P.eps * (div[a] - dadphi[a]) - P.obst * obst - drv;
-        }
-        int na = 0;
-        Real lam = Real(0);
-#pragma unroll
-        for (int a = 0; a < NP; ++a)
+          const Real* fa = s_flux + a * (S::PFX + S::PFY);
+          const Real div = (fa[ty * (BX + 1) + tx + 1] - fa[ty * (BX + 1) + tx]) +
+                           (fa[S::PFX + (ty + 1) * BX + tx] - fa[S::PFX + ty * BX + tx]) + (pfz_hi[a] - pfz_lo[a]);
+          rate[a] = P.eps * (div - dadphi[a]) - P.obst * obst - drv[a];
           if (act & (1u << a)) {
             lam += rate[a];
             ++na;
           }
-        lam = lam / Real(na);
-        Real uv[NP];
-        int m = 0;
+        }
+        lam *= na == 2 ? Real(0.5) : (na == 3 ? Real(1.0 / 3.0) : Real(0.25));
 #pragma unroll
-        for (int a = 0; a < NP; ++a)
-          if (act & (1u << a)) uv[m++] = ph[a] + P.mob_eps * (rate[a] - lam);
-        if (NP == 2) {
-          Real sv = uv[1];
-          sv = sv < Real(0) ? Real(0) : (sv > Real(1) ? Real(1) : sv);
-          out[1] = sv;
-          out[0] = Real(1) - sv;
-        } else {
-          project_simplex<Real, NP>(uv, m);
-          m = 0;
-#pragma unroll
-          for (int a = 0; a < NP; ++a) out[a] = (act & (1u << a)) ? uv[m++] : Real(0);
+        for (int a = 0; a < NP; ++a) out[a] = ph[a] + P.mob_eps * (rate[a] - lam);
+        project_present<NP>(out, act);
         }
       }
     }
@@ -540,7 +621,7 @@ __device__ __forceinline__ void general_tile(const DevParams<Real>& P, const Ste
       bool changed = false;
 #pragma unroll
       for (int a = 0; a < NP; ++a) {
-        s_pn[(slot2(C) * NP + a) * NT + tid] = out[a];
+        if (NP != 2 || a == 1) s_pn[(slot2(C) * NS + (NP == 2 ? 0 : a)) * NT + tid] = out[a];
         changed = changed || out[a] != PH(C, a, r2);
       }
       if constexpr (SHRINK) {
@@ -603,30 +684,18 @@ __device__ __forceinline__ void general_tile(const DevParams<Real>& P, const Ste
         }
         uz_C = u[2];
         if (owner && C >= z0 && C < z0 + ZS && C < P.v_hi) {
+          const PushAxis X = push_axis(gx, nx, P.bc[0] == kWall, 1);
+          const PushAxis Y = push_axis(gy, ny, P.bc[1] == kWall, px);
+          const PushAxis Z = push_axis(C, nz, P.bc[2] == kWall, zst);
           collide<Q>(P, dk, drho, rho, u, F, [&](int k, Real val) {
-            const Store v = Codec<Store>::put(val);
-            int tx_ = gx + Lat::c(k, 0), ty_ = gy + Lat::c(k, 1), tz_ = C + Lat::c(k, 2), kk = k;
-            const bool bx = P.bc[0] == kWall && (tx_ < 0 || tx_ >= nx);
-            const bool by = P.bc[1] == kWall && (ty_ < 0 || ty_ >= ny);
-            const bool bz = P.bc[2] == kWall && (tz_ < 0 || tz_ >= nz);
-            if (bx || by || bz) {  // across a wall the population returns reversed
-              kk = Lat::opp(k);
-              tx_ = gx;
-              ty_ = gy;
-              tz_ = C;
-            } else {
-              tx_ = tx_ < 0 ? tx_ + nx : (tx_ >= nx ? tx_ - nx : tx_);
-              ty_ = ty_ < 0 ? ty_ + ny : (ty_ >= ny ? ty_ - ny : ty_);
-              tz_ = tz_ < 0 ? tz_ + nz : (tz_ >= nz ? tz_ - nz : tz_);
-            }
-            f_out[kk * P.plane + (long long)(tz_ - P.zbase) * zst + (long long)ty_ * px + tx_] = v;
+            push_store<Lat>(f_out, P.plane, gi, k, Codec<Store>::put(val), X, Y, Z);
           });
         }
       }
       s_chg[slot2(C) * NT + tid] = changed ? 1 : 0;
       s_hl[slot2(C) * NT + tid] = interp_h<NP>(out, 0);
 #pragma unroll
-      for (int a = 0; a < NP; ++a) pfz_lo[a] = pfz_hi[a];
+      for (int a = 0; a < NF; ++a) pfz_lo[a] = pfz_hi[a];
     }
     __syncthreads();
 
@@ -639,101 +708,99 @@ __device__ __forceinline__ void general_tile(const DevParams<Real>& P, const Ste
     if (doM) {
       const int fzm = vz(M);
       const bool walls = has_walls;
-      // flux between this cell (plane M) and neighbour nb: d normal axis
-      auto mu_face = [&](int d, int pB, int nbT, int nbR, int gbd, bool obsB, Real* J) {
-        bool closed = (P.bc[d] == kWall && (gbd == 0 || gbd == P.n[d])) || gbd > P.n[d];
-        if (!closed && walls && !lean_d) closed = obstacle(P, fx, fy, fzm) || obsB;
+      // d = 2: the z-face (M, M+1) of this column, for the carry; then, on the
+      // planes it updates, the +x and +y faces into shared memory (one copy of
+      // the code, as for the phase field)
+#pragma unroll
+      for (int f = 0; f < 3; ++f) {
+        if (f > 0 && M == z0 - 1) continue;
+        const int d = f == 0 ? 2 : f - 1;
+        if ((d == 0 && tx >= BX - 1) || (d == 1 && ty >= BY - 1)) continue;
+        const int pB = d == 2 ? M + 1 : M, cB = tid + (d == 0 ? 1 : (d == 1 ? BX : 0));
+        const int rB = r2 + (d == 0 ? 1 : (d == 1 ? W2 : 0));
+        const int gbd = d == 0 ? gx + 1 : (d == 1 ? gy + 1 : M + 1);  // index of B along d
+        const bool wall = d == 0 ? P.bc[0] == kWall : (d == 1 ? P.bc[1] == kWall : P.bc[2] == kWall);
+        const int n = d == 0 ? nx : (d == 1 ? ny : nz);
+        const int fzB = d == 2 ? vz(pB) : fzm;  // vertical index of B (ceq(T))
+        bool closed = (wall && (gbd == 0 || gbd == n)) || gbd > n;
+        if (!closed && walls && !lean_d)
+          closed = obstacle(P, fx, fy, fzm) ||
+                   obstacle(P, d == 0 ? fold_axis(P, gx + 1, 0) : fx, d == 1 ? fold_axis(P, gy + 1, 1) : fy, fzB);
+        Real J[NC];
 #pragma unroll
         for (int i = 0; i < NC; ++i) J[i] = Real(0);
-        if (closed) return;
-        const int pA = M, A = tid, rA = r2;
-        if (lean_d) {
-          const Real ua = d == 2 ? uz_M : s_u[(slot2(pA) * 2 + d) * NT + A];
-          const Real ub = d == 2 ? uz_C : s_u[(slot2(pB) * 2 + d) * NT + nbT];
-          const int fzB = d == 2 ? vz(pB) : fzm;
+        if (!closed) {
+          const Real* mA = s_mu + slot2(M) * NC * NT + tid;
+          const Real* mB = s_mu + slot2(pB) * NC * NT + cB;
+          Real ua = d == 2 ? uz_M : s_u[(slot2(M) * 2 + (d & 1)) * NT + tid];
+          Real ub = d == 2 ? uz_C : s_u[(slot2(pB) * 2 + (d & 1)) * NT + cB];
+          if (lean_d) {
 #pragma unroll
-          for (int i = 0; i < NC; ++i) {
-            const Real ma = s_mu[(slot2(pA) * NC + i) * NT + A], mb = s_mu[(slot2(pB) * NC + i) * NT + nbT];
-            J[i] = liquid_flux(P, ma, mb, ua, ub, ceq_of(0, i, fzm), ceq_of(0, i, fzB));
-          }
-          return;
-        }
-        const Real* pnA = s_pn + slot2(pA) * NP * NT;
-        const Real* pnB = s_pn + slot2(pB) * NP * NT;
-        const Real Mf = Real(0.5) * P.M0 * (pnA[A] + pnB[nbT]);  // plane 0 = liquid
-        const Real ua = (d == 2 ? uz_M : s_u[(slot2(pA) * 2 + d) * NT + A]) * s_hl[slot2(pA) * NT + A];
-        const Real ub = (d == 2 ? uz_C : s_u[(slot2(pB) * 2 + d) * NT + nbT]) * s_hl[slot2(pB) * NT + nbT];
-        const int fzB = d == 2 ? vz(pB) : fzm;  // vertical index of B (ceq(T))
+            for (int i = 0; i < NC; ++i)
+              J[i] = liquid_flux(P, mA[i * NT], mB[i * NT], liquid_adv(P, ua, mA[i * NT], ceq_of(0, i, fzm)),
+                                 liquid_adv(P, ub, mB[i * NT], ceq_of(0, i, fzB)));
+          } else {
+            // no liquid in either cell before or after the step: M, h_l and the
+            // liquid weight of the antitrapping current are 0, and J with them
+            const Real la = PN(M, 0, tid), lb = PN(pB, 0, cB);
+            const Real lf = Real(0.5) * (PH(M, 0, r2) + PH(pB, 0, rB));
+            if (la + lb + lf != Real(0)) {
+              const Real Mf = Real(0.5) * P.M0 * (la + lb);
+              ua *= s_hl[slot2(M) * NT + tid];
+              ub *= s_hl[slot2(pB) * NT + cB];
 #pragma unroll
-        for (int i = 0; i < NC; ++i) {
-          const Real ma = s_mu[(slot2(pA) * NC + i) * NT + A], mb = s_mu[(slot2(pB) * NC + i) * NT + nbT];
-          J[i] = -Mf * (mb - ma) + Real(0.5) * (ua * (ceq_of(0, i, fzm) + ma * P.inv2A[0]) +
-                                                ub * (ceq_of(0, i, fzB) + mb * P.inv2A[0]));
-        }
-        // the current carries phi_l's face value as a factor of every term: on
-        // a face without liquid (grain boundaries inside the solid) it is
-        // exactly 0 and skipped
-        const Real liq = P.at_eps != Real(0) && (s_chg[slot2(pA) * NT + A] | s_chg[slot2(pB) * NT + nbT])
-                             ? Real(0.5) * (PH(pA, 0, rA) + PH(pB, 0, nbR))
-                             : Real(0);
-        if (liq != Real(0)) {
-          Real at[NC];
+              for (int i = 0; i < NC; ++i) {
+                const Real ma = mA[i * NT], mb = mB[i * NT];
+                J[i] = -Mf * (mb - ma) + Real(0.5) * (ua * (ceq_of(0, i, fzm) + ma * P.inv2A[0]) +
+                                                      ub * (ceq_of(0, i, fzB) + mb * P.inv2A[0]));
+              }
+              // the antitrapping current carries phi_l's face value as a factor
+              // of every term
+              const bool moves = P.at_eps != Real(0) && (s_chg[slot2(M) * NT + tid] | s_chg[slot2(pB) * NT + cB]);
+              if (moves && lf != Real(0)) {
+                auto at = [&](int p, int i) { return slot4(p) * NS * C2 + i; };
+                const int A = at(M, r2), B = at(pB, rB), st = d == 0 ? W2 : 1;
+                const int ap = d == 2 ? A + W2 : at(M + 1, r2), am = d == 2 ? A - W2 : at(M - 1, r2);
+                const int bp = d == 2 ? B + W2 : at(M + 1, rB), bm = d == 2 ? B - W2 : at(M - 1, rB);
+                Real trap[NC];
 #pragma unroll
-          for (int i = 0; i < NC; ++i) at[i] = Real(0);
+                for (int i = 0; i < NC; ++i) trap[i] = Real(0);
 #pragma unroll
-          for (int a = 1; a < NP; ++a) {
-            const Real va = PH(pA, a, rA), vb = PH(pB, a, nbR);
-            const Real gn = vb - va;
-            Real t1, t2;
-            if (d == 2) {
-              t1 = Real(0.25) * (PH(pA, a, rA + 1) + PH(pB, a, nbR + 1) - PH(pA, a, rA - 1) - PH(pB, a, nbR - 1));
-              t2 = Real(0.25) * (PH(pA, a, rA + W2) + PH(pB, a, nbR + W2) - PH(pA, a, rA - W2) - PH(pB, a, nbR - W2));
-            } else {
-              const int st = d == 0 ? W2 : 1;
-              t1 = Real(0.25) * (PH(pA, a, rA + st) + PH(pB, a, nbR + st) - PH(pA, a, rA - st) - PH(pB, a, nbR - st));
-              t2 = Real(0.25) * (PH(pA + 1, a, rA) + PH(pB + 1, a, nbR) - PH(pA - 1, a, rA) - PH(pB - 1, a, nbR));
-            }
-            const Real g2 = gn * gn + t1 * t1 + t2 * t2;
-            if (g2 <= Real(1e-12)) continue;
-            const Real nd = liq * gn / sqrt(g2);
-            const Real dphi = Real(0.5) * ((pnA[a * NT + A] - va) + (pnB[a * NT + nbT] - vb));
-            const Real dinv = P.inv2A[0] - P.inv2A[a];
+                for (int a = 1; a < NP; ++a) {
+                  const Real* ph = s_phi + (NP == 2 ? 0 : a) * C2;
+                  const Real va = ph[A], vb = ph[B], gn = vb - va;
+                  const Real t1 = Real(0.25) * (ph[A + st] + ph[B + st] - ph[A - st] - ph[B - st]);
+                  const Real t2 = Real(0.25) * (ph[ap] + ph[bp] - ph[am] - ph[bm]);
+                  const Real g2 = gn * gn + t1 * t1 + t2 * t2;
+                  if (g2 <= Real(1e-12)) continue;
+                  const Real nd = lf * gn / sqrt(g2);
+                  const Real dphi = Real(0.5) * ((PN(M, a, tid) - va) + (PN(pB, a, cB) - vb));
+                  const Real dinv = P.inv2A[0] - P.inv2A[a];
 #pragma unroll
-            for (int i = 0; i < NC; ++i) {
-              Real dc = (P.ceq[0][i] - P.ceq[a][i]) +
-                        Real(0.5) * (s_mu[(slot2(pA) * NC + i) * NT + A] + s_mu[(slot2(pB) * NC + i) * NT + nbT]) * dinv;
-              if constexpr (EXT)
-                dc += (P.dceq_dT[0][i] - P.dceq_dT[a][i]) * (theta_base + Real(0.5) * P.G * Real(fzm + fzB));
-              at[i] += dc * dphi * nd;
+                  for (int i = 0; i < NC; ++i) {
+                    Real dc = (P.ceq[0][i] - P.ceq[a][i]) + Real(0.5) * (mA[i * NT] + mB[i * NT]) * dinv;
+                    if constexpr (EXT)
+                      dc += (P.dceq_dT[0][i] - P.dceq_dT[a][i]) * (theta_base + Real(0.5) * P.G * Real(fzm + fzB));
+                    trap[i] += dc * dphi * nd;
+                  }
+                }
+#pragma unroll
+                for (int i = 0; i < NC; ++i) J[i] -= P.at_eps * trap[i];
+              }
             }
           }
-#pragma unroll
-          for (int i = 0; i < NC; ++i) J[i] -= P.at_eps * at[i];
         }
-      };
-      // z-face (M, M+1) of this column, for the carry
-      {
-        const int fzb = vz(M + 1);
-        mu_face(2, M + 1, tid, r2, M + 1, walls && !lean_d && obstacle(P, fx, fy, fzb), mz_hi);
+        if (d == 2) {
+#pragma unroll
+          for (int i = 0; i < NC; ++i) mz_hi[i] = J[i];
+        } else {
+#pragma unroll
+          for (int i = 0; i < NC; ++i) s_flux[(i * 2 + d) * NT + tid] = J[i];
+        }
       }
       if (M == z0 - 1) {
 #pragma unroll
         for (int i = 0; i < NC; ++i) mz_lo[i] = mz_hi[i];
-      } else {
-        // in-plane faces of plane M
-        Real J[NC];
-        if (tx < BX - 1) {
-          const bool ob = walls && !lean_d && obstacle(P, fold_axis(P, gx + 1, 0), fy, fzm);
-          mu_face(0, M, tid + 1, r2 + 1, gx + 1, ob, J);
-#pragma unroll
-          for (int i = 0; i < NC; ++i) s_flux[(i * 2 + 0) * NT + tid] = J[i];
-        }
-        if (ty < BY - 1) {
-          const bool ob = walls && !lean_d && obstacle(P, fx, fold_axis(P, gy + 1, 1), fzm);
-          mu_face(1, M, tid + BX, r2 + W2, gy + 1, ob, J);
-#pragma unroll
-          for (int i = 0; i < NC; ++i) s_flux[(i * 2 + 1) * NT + tid] = J[i];
-        }
       }
     }
     __syncthreads();
@@ -744,7 +811,7 @@ __device__ __forceinline__ void general_tile(const DevParams<Real>& P, const Ste
 #pragma unroll
       for (int a = 0; a < NP; ++a) {
         po[a] = PH(M, a, r2);
-        pn[a] = s_pn[(slot2(M) * NP + a) * NT + tid];
+        pn[a] = PN(M, a, tid);
       }
 #pragma unroll
       for (int sidx = 0; sidx < NS; ++sidx) phi_out[sidx * P.plane + g] = pn[NP == 2 ? 1 : sidx];
@@ -782,6 +849,24 @@ __device__ __forceinline__ void general_tile(const DevParams<Real>& P, const Ste
           const Real div = (Jx[tid] - Jx[tid - 1]) + (Jy[tid] - Jy[tid - BX]) + (mz_hi[i] - mz_lo[i]);
           const Real mu = s_mu[(slot2(M) * NC + i) * NT + tid];
           mu_out[i * P.plane + g] = mu + (-div - Real(0)) * ichi;
+        }
+      } else if constexpr (NP == 2) {
+        // h_0 = 1 - h_1: chi and the source need h_1 alone
+        auto h1 = [](Real v) { return v * v * (Real(3) - Real(2) * v); };
+        const Real dinv = P.inv2A[1] - P.inv2A[0], hn = h1(pn[1]);
+        // (the same A in both phases: chi = 1 / (2 A))
+        const Real ichi = is_zero(dinv) ? P.chi_pure[0] : rcp_rn(P.inv2A[0] + hn * dinv);
+        const Real dh = s_chg[slot2(M) * NT + tid] != 0 ? hn - h1(po[1]) : Real(0);
+#pragma unroll
+        for (int i = 0; i < NC; ++i) {
+          const Real* Jx = s_flux + (i * 2 + 0) * NT;
+          const Real* Jy = s_flux + (i * 2 + 1) * NT;
+          const Real div = (Jx[tid] - Jx[tid - 1]) + (Jy[tid] - Jy[tid - BX]) + (mz_hi[i] - mz_lo[i]);
+          const Real mu = s_mu[(slot2(M) * NC + i) * NT + tid];
+          Real src = ((ceq_of(1, i, fzm) - ceq_of(0, i, fzm)) + mu * dinv) * dh;
+          // -(dT/dt) sum_a (dc_a/dT)_mu h_a^{n+1}, dT/dt = -G V
+          if constexpr (EXT) src -= P.GV_r * (P.dceq_dT[0][i] + (P.dceq_dT[1][i] - P.dceq_dT[0][i]) * hn);
+          mu_out[i * P.plane + g] = mu + (-div - src) * ichi;
         }
       } else {
         Real chi = Real(0), hn[NP], ho[NP];

@@ -4,7 +4,7 @@
 // in every 3x3x3 neighbourhood, so it has no rate), the chemical potential
 // diffusing with M = D_liq / (2 A_l) and advected by U^n with h_l = 1 and
 // chi = 1 / (2 A_l), and the lattice Boltzmann step with phi_l = 1 (no drag,
-// the full buoyancy).  liquid_tile advances such tiles with the same
+// the full buoyancy).  liquid_march advances such tiles with the same
 // arithmetic, term for term, as the general path's liquid planes --
 // the results are bit-identical -- but without the phase-field machinery,
 // so it needs far fewer registers and instructions.
@@ -22,32 +22,49 @@
 
 namespace gpflbm {
 
+// Segments one CTA of the liquid path may march in one go.  A march repeats two
+// planes, 8 for the 6 of one segment and 14 for 12.  With 16-bit populations
+// the path is bound by instruction issue and marches two (FP16 dendrite 256^3:
+// 603 us a step against 638); with FP32 ones by the traffic between L2 and the
+// SMs, where the z-neighbours' planes are in L2 more often the sooner they are
+// read again, and marches one (ternary eutectic: 1.65 ms against 1.73 with two,
+// 1.83 with three).
+template <class Store>
+constexpr int kLiquidGroup = sizeof(Store) == 2 ? 2 : 1;
+
 template <int NP, int NC, class Real, class Store, int QQ = 19, bool EXT = false>
 struct Liquid3D {
   static constexpr int BX = Block3D<Real>::BX, BY = Block3D<Real>::BY, ZS = Block3D<Real>::ZS;
   static constexpr int NT = BX * BY;
   static constexpr int OX = BX - 2, OY = BY - 2;
-  static constexpr size_t al(size_t v) { return (v + 15) / 16 * 16; }
-  // a ring of three planes of U and mu, and the in-plane solute fluxes of
-  // two planes: one barrier a plane (see liquid_tile)
-  static constexpr size_t u = 0;                                    // 3 planes x 3 x NT
-  static constexpr size_t mu = al(u + sizeof(Real) * 3 * 3 * NT);   // 3 planes x NC x NT
-  static constexpr size_t flux = al(mu + sizeof(Real) * 3 * NC * NT);  // 2 planes x 2 x NC x NT
-  static constexpr size_t bytes = al(flux + sizeof(Real) * 2 * 2 * NC * NT);
+  // mu and the y current of a plane, for the rows next to a thread's (its own
+  // row is its warp, its own column its registers), in two slots: one barrier
+  // a plane
+  static constexpr size_t bytes = sizeof(Real) * 2 * 2 * NC * NT;
 };
 
-// The liquid path for one tile (coordinates as for general_tile).
+// The liquid path for n planes from z0 of xy tile (bx, by) (z0 + n <= v_hi).
+// Bound by the sectors that pass between L2 and the SMs and by instruction
+// issue: a kernel that only loads and stores the 21 planes of the ternary
+// eutectic in this pattern takes 1.26 ms for 256 x 256 x 512 cells (6.8 TB/s
+// without halos and off-by-one rows: 0.85 ms), this path 1.24 ms.  x-faces pass
+// between the lanes of a warp (a warp is a row of the tile), z-faces stay in a
+// thread's registers, and each thread forms both its y-faces, so that shared
+// memory holds mu and the y currents alone.  A cell mirrored at a wall hands
+// out its currents with the sign turned, which makes the flux through the
+// wall's face exactly zero without a test.
 template <int NP, int NC, class Real, class Store, int QQ, bool EXT>
-__device__ __forceinline__ void liquid_tile(const DevParams<Real>& P, const Step3DIO& io, int bx, int by, int bz,
-                                            int gxt, int gyt) {
+__device__ __forceinline__ void liquid_march(const DevParams<Real>& P, const Step3DIO& io, int bx, int by, int z0,
+                                             int n, int gxt, int gyt) {
   using S = Liquid3D<NP, NC, Real, Store, QQ, EXT>;
   using Lat = Lattice<QQ>;
-  constexpr int BX = S::BX, BY = S::BY, ZS = S::ZS, NT = S::NT, Q = QQ;
+  constexpr int BX = S::BX, BY = S::BY, NT = S::NT, Q = QQ;
   constexpr int NS = PhiStore<NP>::NS;
+  static_assert(BX == 32, "a row of the tile is a warp");
   extern __shared__ __align__(16) unsigned char smem[];
-  Real* s_u = reinterpret_cast<Real*>(smem + S::u);
-  Real* s_mu = reinterpret_cast<Real*>(smem + S::mu);
-  Real* s_flux = reinterpret_cast<Real*>(smem + S::flux);
+  // planes whose phi in the output buffer already is pure liquid (its flags,
+  // from when it was last written): nothing to write there
+  __shared__ unsigned char s_have[kLiquidGroup<Store> * S::ZS];
 
   const Real* __restrict__ mu_in = static_cast<const Real*>(io.mu_in);
   const Store* __restrict__ f_in = static_cast<const Store*>(io.f_in);
@@ -59,58 +76,61 @@ __device__ __forceinline__ void liquid_tile(const DevParams<Real>& P, const Step
   const int tx = tid % BX, ty = tid / BX;
   const int nx = P.n[0], ny = P.n[1], nz = P.n[2], px = P.px;
   const int zst = px * ny;
-  const int x0 = bx * S::OX, y0 = by * S::OY, z0 = P.v_lo + bz * ZS;
+  const int x0 = bx * S::OX, y0 = by * S::OY;
   const int gx = x0 - 1 + tx, gy = y0 - 1 + ty;
+  // (tiles this far inside are the general path's: one condition for both)
   const bool inner_xy = x0 >= 2 && x0 - 2 + BX + 2 <= nx && y0 >= 2 && y0 - 2 + BY + 2 <= ny;
   const int fx = inner_xy ? gx : fold_axis(P, gx, 0);
   const int fy = inner_xy ? gy : fold_axis(P, gy, 1);
   const int gxy = fy * px + fx;
   const bool owner = tx >= 1 && tx <= BX - 2 && ty >= 1 && ty <= BY - 2 && gx < nx && gy < ny;
-  const double t_now = io.clock_in[0];
-  if (bx == 0 && by == 0 && bz == 0 && tid == 0) io.clock_out[0] = t_now + 1.0;
-  const Real theta_base = theta_at(P, t_now);
-  auto ceq_of = [&](int a, int i, int v) -> Real {
+  if (tid < n) s_have[tid] = io.flags_out[liquid_flag_index(bx, by, z0 + tid, gxt, gyt)];
+  const Real theta_base = theta_at(P, io.clock_in[0]);
+  auto ceq_of = [&](int i, int v) -> Real {
     if constexpr (EXT)
-      return fma_rn(P.dceq_dT[a][i], fma_rn(P.G, Real(v), theta_base), P.ceq[a][i]);
+      return fma_rn(P.dceq_dT[0][i], fma_rn(P.G, Real(v), theta_base), P.ceq[0][i]);
     else
-      return P.ceq[a][i];
+      return P.ceq[0][i];
   };
+  // planes z0 - 1 .. z0 + n, folded at the ends of the vertical axis
+  const bool zin = z0 >= 1 && z0 + n < nz;
   auto vz = [&](int v) {
+    if (zin) return v;
     const int f = fold_axis(P, v, 2);
     return f < P.v_lo - 2 ? P.v_lo - 2 : (f > P.v_hi + 1 ? P.v_hi + 1 : f);
   };
   auto zrow = [&](int fz) { return (fz - P.zbase) * zst; };
-  // the segment and its two halo planes lie inside the grid: no folding and
-  // no closed z-face (in-plane faces of an inner tile are never closed)
-  const bool zin = z0 >= 1 && z0 + ZS <= nz - 1;
-  auto vzi = [&](int v) { return zin ? v : vz(v); };
+  // a cell mirrored at a wall in x, y
+  const bool mirror_x = P.bc[0] == kWall && (gx < 0 || gx >= nx);
+  const bool mirror_y = P.bc[1] == kWall && (gy < 0 || gy >= ny);
+  const int up = ty < BY - 1 ? BX : 0, down = ty > 0 ? -BX : 0;
 
-  // solute z-face fluxes of this column: (M-1, M) carried, (M, M+1) new
-  Real mz_lo[NC], mz_hi[NC];
+  Store fk[Q];
+  Real mu_n[NC];
+  auto load = [&](int v) {
+    const int g = zrow(vz(v)) + gxy;
 #pragma unroll
-  for (int i = 0; i < NC; ++i) mz_lo[i] = mz_hi[i] = Real(0);
-
-  // Ring slots of planes M and C = M + 1.  One barrier a plane: the in-plane
-  // fluxes of a plane are formed in the iteration that produced its U and
-  // mu, into one half of a double buffer, and read by the next iteration's
-  // update; three slots of U and mu, so that the slot B overwrites held the
-  // plane three back, which no thread reads after the previous barrier.
-  int sM = 2, sC = 0;
-  for (int C = z0 - 1; C <= z0 + ZS; ++C) {
-    const int M = C - 1;
-    // B. moments, U and (owned planes) collision + push, plane C
+    for (int k = 0; k < Q; ++k) fk[k] = at_bytes(f_in + g, P.f_at[k]);
+#pragma unroll
+    for (int i = 0; i < NC; ++i) mu_n[i] = (mu_in + i * P.plane)[g];
+  };
+  // of the plane below: mu and the z current of this column, the in-plane part
+  // of the divergence, and the solute flux through its lower z-face
+  Real mu_b[NC], wz_b[NC], div_b[NC], z_lo[NC];
+#pragma unroll
+  for (int i = 0; i < NC; ++i) mu_b[i] = wz_b[i] = div_b[i] = z_lo[i] = Real(0);
+  for (int C = z0 - 1; C <= z0 + n; ++C) {
+    const bool inside = C >= z0 && C < z0 + n;  // a plane this march advances
+    const int fzc = vz(C), gi = zrow(fzc) + gxy;
+    Real* const sl = reinterpret_cast<Real*>(smem) + (C & 1) * 2 * NC * NT + tid;
+    Real mu[NC], wx[NC], wy[NC], wz[NC];
     {
-      const int fzc = vzi(C);
-      const int gi = zrow(fzc) + gxy;
-      Real mu[NC];
-#pragma unroll
-      for (int i = 0; i < NC; ++i) {
-        mu[i] = (mu_in + i * P.plane)[gi];
-        s_mu[(sC * NC + i) * NT + tid] = mu[i];
-      }
       Real dk[Q];
+      load(C);
 #pragma unroll
-      for (int k = 0; k < Q; ++k) dk[k] = Codec<Store>::load(at_bytes(f_in + gi, P.f_at[k]));
+      for (int k = 0; k < Q; ++k) dk[k] = Codec<Store>::load(fk[k]);
+#pragma unroll
+      for (int i = 0; i < NC; ++i) mu[i] = mu_n[i];
       Real drho = Real(0), m3[3] = {Real(0), Real(0), Real(0)};
 #pragma unroll
       for (int k = 0; k < Q; ++k) {
@@ -120,107 +140,138 @@ __device__ __forceinline__ void liquid_tile(const DevParams<Real>& P, const Step
           if (Lat::c(k, a) != 0) m3[a] += Real(Lat::c(k, a)) * dk[k];
       }
       const Real rho = Real(1) + drho;
-      // the general path's arithmetic with phi_l = 1 (the same helpers)
-      const Real drive = buoyancy_drive<NC, EXT>(P, fma_rn(P.G, Real(fzc), theta_base), mu);
-      Real u[3], F[3];
-      force_velocity<3>(P, rho, Real(1), drive, m3, u, F);
+      // force_velocity with phi_l = 1: no drag, the buoyancy alone
+      const Real FB = mul_rn(rho, buoyancy_drive<NC, EXT>(P, fma_rn(P.G, Real(fzc), theta_base), mu));
+      const Real inv = rcp_rn(rho);
+      const Real u[3] = {mul_rn(m3[0], inv), mul_rn(m3[1], inv), mul_rn(fma_rn(Real(0.5), FB, m3[2]), inv)};
 #pragma unroll
-      for (int a = 0; a < 3; ++a) s_u[(sC * 3 + a) * NT + tid] = u[a];
-      if (owner && C >= z0 && C < z0 + ZS && C < P.v_hi) {
-        const bool inner_z = C >= 1 && C + 1 < nz;
-        if (inner_xy && inner_z) {
+      for (int i = 0; i < NC; ++i) {
+        const Real c = ceq_of(i, fzc);
+        wx[i] = liquid_adv(P, u[0], mu[i], c);
+        wy[i] = liquid_adv(P, u[1], mu[i], c);
+        wz[i] = liquid_adv(P, u[2], mu[i], c);
+        if (mirror_x) wx[i] = -wx[i];
+        if (mirror_y) wy[i] = -wy[i];
+      }
+      if (inside) {
+#pragma unroll
+        for (int i = 0; i < NC; ++i) {
+          sl[(2 * i) * NT] = mu[i];
+          sl[(2 * i + 1) * NT] = wy[i];
+        }
+      }
+      if (owner && inside) {
+        const Real F[3] = {Real(0), Real(0), FB};
+        if (inner_xy && C >= 1 && C + 1 < nz) {
           Store* const fo = f_out + gi;
-          collide<Q>(P, dk, drho, rho, u, F, [&](int k, Real val) { at_bytes(fo, P.f_to[k]) = Codec<Store>::put(val); });
+          collide<Q, true>(P, dk, drho, rho, u, F,
+                           [&](int k, Real val) { at_bytes(fo, P.f_to[k]) = Codec<Store>::put(val); });
         } else {
           const PushAxis X = push_axis(gx, nx, P.bc[0] == kWall, 1);
           const PushAxis Y = push_axis(gy, ny, P.bc[1] == kWall, px);
           const PushAxis Z = push_axis(C, nz, P.bc[2] == kWall, zst);
-          collide<Q>(P, dk, drho, rho, u, F, [&](int k, Real val) {
+          collide<Q, true>(P, dk, drho, rho, u, F, [&](int k, Real val) {
             push_store<Lat>(f_out, P.plane, gi, k, Codec<Store>::put(val), X, Y, Z);
           });
         }
       }
     }
-    __syncthreads();
-    // D. solute fluxes (every plane M-1 .. C+1 liquid: M = M0, h_l = 1).
-    // face between this cell in plane pA (slot sA) and nbT in plane pB (slot sB)
-    auto face = [&](int d, int pA, int sA, int pB, int sB, int nbT, int gbd, Real* J) {
-      const bool open = d == 2 ? zin : inner_xy;
-      const bool closed = !open && ((P.bc[d] == kWall && (gbd == 0 || gbd == P.n[d])) || gbd > P.n[d]);
+    if (inside) __syncthreads();
+    if (C >= z0) {
+      // the z-face between this plane and the one below, whose update it ends
+      const int M = C - 1;
+      const bool closed = !zin && P.bc[2] == kWall && (C == 0 || C == nz);
+      Real z_hi[NC];
 #pragma unroll
-      for (int i = 0; i < NC; ++i) J[i] = Real(0);
-      if (closed) return;
-      const int fzA = vzi(pA);
-      const Real ua = s_u[(sA * 3 + d) * NT + tid], ub = s_u[(sB * 3 + d) * NT + nbT];
-      const int fzB = d == 2 ? vzi(pB) : fzA;
+      for (int i = 0; i < NC; ++i) z_hi[i] = closed ? Real(0) : liquid_flux(P, mu_b[i], mu[i], wz_b[i], wz[i]);
+      if (M >= z0 && owner) {
+        const int g = zrow(M) + gxy;
+        if (!s_have[M - z0]) {
 #pragma unroll
-      for (int i = 0; i < NC; ++i) {
-        const Real ma = s_mu[(sA * NC + i) * NT + tid], mb = s_mu[(sB * NC + i) * NT + nbT];
-        J[i] = liquid_flux(P, ma, mb, ua, ub, ceq_of(0, i, fzA), ceq_of(0, i, fzB));
-      }
-    };
-    // the z-face (M, C) of this column
-    const bool doM = M >= z0 - 1 && M <= z0 + ZS - 1;
-    if (doM) {
-      face(2, M, sM, C, sC, tid, C, mz_hi);
-      if (M == z0 - 1) {
-#pragma unroll
-        for (int i = 0; i < NC; ++i) mz_lo[i] = mz_hi[i];
-      }
-    }
-    // the update of plane M: its in-plane fluxes (formed last iteration) and
-    // its two z-faces
-    if (doM && M >= z0 && M < P.v_hi && owner) {
-      const Real* fl = s_flux + (M & 1) * 2 * NC * NT;
-      const int g = zrow(M) + gxy;
-#pragma unroll
-      for (int sidx = 0; sidx < NS; ++sidx)
-        phi_out[sidx * P.plane + g] = (NP != 2 && sidx == 0) ? Real(1) : Real(0);
-#pragma unroll
-      for (int i = 0; i < NC; ++i) {
-        const Real* Jx = fl + (i * 2 + 0) * NT;
-        const Real* Jy = fl + (i * 2 + 1) * NT;
-        const Real div = (Jx[tid] - Jx[tid - 1]) + (Jy[tid] - Jy[tid - BX]) + (mz_hi[i] - mz_lo[i]);
-        const Real mu = s_mu[(sM * NC + i) * NT + tid];
-        Real src = Real(0);
-        if constexpr (EXT) {
-#pragma unroll
-          for (int a = 0; a < NP; ++a) src -= P.GV_r * P.dceq_dT[a][i] * (a == 0 ? Real(1) : Real(0));
+          for (int sidx = 0; sidx < NS; ++sidx)
+            phi_out[sidx * P.plane + g] = (NP != 2 && sidx == 0) ? Real(1) : Real(0);
         }
-        mu_out[i * P.plane + g] = liquid_mu(P, mu, div, src);
+#pragma unroll
+        for (int i = 0; i < NC; ++i) {
+          const Real div = div_b[i] + sub_rn(z_hi[i], z_lo[i]);
+          Real src = Real(0);
+          if constexpr (EXT) {
+#pragma unroll
+            for (int a = 0; a < NP; ++a) src -= P.GV_r * P.dceq_dT[a][i] * (a == 0 ? Real(1) : Real(0));
+          }
+          mu_out[i * P.plane + g] = liquid_mu(P, mu_b[i], div, src);
+        }
+      }
+#pragma unroll
+      for (int i = 0; i < NC; ++i) z_lo[i] = z_hi[i];
+    }
+    if (inside) {
+#pragma unroll
+      for (int i = 0; i < NC; ++i) {
+        const Real* m = sl + (2 * i) * NT;
+        const Real* w = sl + (2 * i + 1) * NT;
+        const Real mr = __shfl_down_sync(0xffffffffu, mu[i], 1), wr = __shfl_down_sync(0xffffffffu, wx[i], 1);
+        const Real jr = liquid_flux(P, mu[i], mr, wx[i], wr);
+        const Real jl = __shfl_up_sync(0xffffffffu, jr, 1);
+        const Real ju = liquid_flux(P, mu[i], m[up], wy[i], w[up]);
+        const Real jd = liquid_flux(P, m[down], mu[i], w[down], wy[i]);
+        div_b[i] = sub_rn(jr, jl) + sub_rn(ju, jd);
       }
     }
-    if (doM && M >= z0) {
 #pragma unroll
-      for (int i = 0; i < NC; ++i) mz_lo[i] = mz_hi[i];
+    for (int i = 0; i < NC; ++i) {
+      mu_b[i] = mu[i];
+      wz_b[i] = wz[i];
     }
-    // the in-plane fluxes of plane C, for its update in the next iteration
-    if (C >= z0 && C <= z0 + ZS - 1) {
-      Real* fl = s_flux + (C & 1) * 2 * NC * NT;
-      Real J[NC];
-      if (tx < BX - 1) {
-        face(0, C, sC, C, sC, tid + 1, gx + 1, J);
-#pragma unroll
-        for (int i = 0; i < NC; ++i) fl[(i * 2 + 0) * NT + tid] = J[i];
-      }
-      if (ty < BY - 1) {
-        face(1, C, sC, C, sC, tid + BX, gy + 1, J);
-#pragma unroll
-        for (int i = 0; i < NC; ++i) fl[(i * 2 + 1) * NT + tid] = J[i];
-      }
-    }
-    sM = sC;
-    sC = sC == 2 ? 0 : sC + 1;
   }
-  if (tid < ZS && z0 + tid < P.v_hi) io.flags_out[liquid_flag_index(bx, by, z0 + tid, gxt, gyt)] = 1;
+  if (tid < n) io.flags_out[liquid_flag_index(bx, by, z0 + tid, gxt, gyt)] = 1;
+}
+
+// The liquid tiles of the group of segments starting at segment bz of xy tile
+// (bx, by): each run of neighbouring liquid segments is one march.  Which
+// segments are liquid is decided as the general pass decides it
+// (liquid_reach).
+template <int NP, int NC, class Real, class Store, int QQ, bool EXT>
+__device__ __forceinline__ void liquid_tiles(const DevParams<Real>& P, const Step3DIO& io, int bx, int by, int bz,
+                                             int gxt, int gyt) {
+  using S = Liquid3D<NP, NC, Real, Store, QQ, EXT>;
+  constexpr int ZS = S::ZS, G = kLiquidGroup<Store>;
+  static_assert(9 * (G * ZS + 4) <= S::NT, "one flag a thread");
+  __shared__ int s_bad[G];
+  const int z0 = P.v_lo + bz * ZS, group = P.liq_group;
+  const int tid = threadIdx.x;
+  if (bx == 0 && by == 0 && bz == 0 && tid == 0) io.clock_out[0] = io.clock_in[0] + 1.0;
+  if (tid < G) s_bad[tid] = 0;
+  __syncthreads();
+  if (tid < 9 * (group * ZS + 4)) {
+    const int p = tid / 9;
+    if (!liquid_flag_near(P, io.flags_in, bx, by, z0 - 2 + p, tid - 9 * p, gxt, gyt)) {
+#pragma unroll
+      for (int s = 0; s < G; ++s)
+        if (s < group && p >= s * ZS && p < s * ZS + ZS + 4) s_bad[s] = 1;
+    }
+  }
+  __syncthreads();
+  for (int s = 0; s < group && z0 + s * ZS < P.v_hi;) {
+    if (s_bad[s]) {
+      ++s;
+      continue;
+    }
+    int e = s + 1;
+    while (e < group && z0 + e * ZS < P.v_hi && !s_bad[e]) ++e;
+    const int zs = z0 + s * ZS, ze = min(z0 + e * ZS, P.v_hi);
+    liquid_march<NP, NC, Real, Store, QQ, EXT>(P, io, bx, by, zs, ze - zs, gxt, gyt);
+    __syncthreads();  // (s_have and the slots are reused)
+    s = e;
+  }
 }
 
 // The step kernels.  Where both paths fit 64 registers (FP32 arithmetic on
 // D3Q19: two CTAs share an SM either way) and the general path is that of
 // two phases (Step3D::ONE_LAUNCH), one launch takes every tile: its
-// grid holds the tiling twice, z blocks 0 .. gzt-1 the general pass and
-// gzt .. 2 gzt-1 the liquid pass, and a CTA returns unless its tile's flags
-// pick its pass.  CTAs start in block order, so the general tiles, the slow
+// grid holds the tiling twice, z blocks 0 .. gzt-1 the general pass and those
+// after them the liquid pass (a group of segments each), and a CTA returns
+// unless its tile's flags pick its pass.  CTAs start in block order, so the general tiles, the slow
 // ones, start first and the liquid tiles fill the SMs as they finish
 // instead of waiting for the last general tile.  Elsewhere (FP64, D3Q27:
 // the general path needs more registers than the liquid one, and one kernel
@@ -235,24 +286,22 @@ __global__ void __launch_bounds__(Step3D<NP, NC, Real, Store, QQ>::NT, Step3D<NP
   const int gxt = gridDim.x, gyt = gridDim.y, gzt = (P.v_hi - P.v_lo + ZS - 1) / ZS;
   const int bx = blockIdx.x, by = blockIdx.y;
   const bool liquid_pass = S::ONE_LAUNCH && (int)blockIdx.z >= gzt;
-  const int bz = liquid_pass ? (int)blockIdx.z - gzt : (int)blockIdx.z;
-  if (P.liq_dispatch && liquid_reach<ZS>(P, io.flags_in, bx, by, P.v_lo + bz * ZS, gxt, gyt) != liquid_pass) return;
   if constexpr (S::ONE_LAUNCH) {
     if (liquid_pass) {
-      liquid_tile<NP, NC, Real, Store, QQ, EXT>(P, io, bx, by, bz, gxt, gyt);
+      liquid_tiles<NP, NC, Real, Store, QQ, EXT>(P, io, bx, by, ((int)blockIdx.z - gzt) * P.liq_group, gxt, gyt);
       return;
     }
   }
+  const int bz = blockIdx.z;
+  if (P.liq_dispatch && liquid_reach<ZS>(P, io.flags_in, bx, by, P.v_lo + bz * ZS, gxt, gyt)) return;
   general_tile<NP, NC, Real, Store, SHRINK, QQ, EXT>(P, io, bx, by, bz, gxt, gyt);
 }
 
 template <int NP, int NC, class Real, class Store, int QQ = 19, bool EXT = false>
 __global__ void __launch_bounds__(Liquid3D<NP, NC, Real, Store, QQ, EXT>::NT, 2)
     step3d_liquid_kernel(const DevParams<Real> P, const Step3DIO io) {
-  constexpr int ZS = Liquid3D<NP, NC, Real, Store, QQ, EXT>::ZS;
-  if (!liquid_reach<ZS>(P, io.flags_in, blockIdx.x, blockIdx.y, P.v_lo + blockIdx.z * ZS, gridDim.x, gridDim.y))
-    return;
-  liquid_tile<NP, NC, Real, Store, QQ, EXT>(P, io, blockIdx.x, blockIdx.y, blockIdx.z, gridDim.x, gridDim.y);
+  liquid_tiles<NP, NC, Real, Store, QQ, EXT>(P, io, blockIdx.x, blockIdx.y, blockIdx.z * P.liq_group, gridDim.x,
+                                             gridDim.y);
 }
 
 // The liquid flags of a state (after a load or a frame shift): one CTA per
