@@ -176,8 +176,12 @@ struct Impl {
       const unsigned gz = (P.v_hi - P.v_lo + S3::ZS - 1) / S3::ZS;
       const dim3 grid((P.n[0] + S3::OX - 1) / S3::OX, (P.n[1] + S3::OY - 1) / S3::OY,
                       S3::ONE_LAUNCH && P.liq_dispatch ? gz + (gz + P.liq_group - 1) / P.liq_group : gz);
-      const Step3DIO sio = {io.phi_in, io.phi_out, io.mu_in,    io.mu_out,    io.f_in,
+      Step3DIO sio = {io.phi_in, io.phi_out, io.mu_in,    io.mu_out,    io.f_in,
                       io.f_out,  io.clock_in, io.clock_out, io.flags_in, io.flags_out};
+      for (int k = 0; k < Q; ++k) {
+        sio.fi[k] = static_cast<const char*>(io.f_in) + P.f_at[k];
+        sio.fo[k] = static_cast<char*>(io.f_out) + P.f_to[k];
+      }
       if (P.shrink)
         step3d_kernel<NP, NC, Real, Store, true, Q, EXT><<<grid, S3::NT, step3d_bytes, s>>>(P, sio);
       else

@@ -90,6 +90,10 @@ struct Step3DIO {
   double* clock_out;
   const unsigned char* flags_in;  // liquid flag per tile of the input state
   unsigned char* flags_out;       // ... of the output state
+  // population k of cell 0, and where its collided population k lands (f_at,
+  // f_to added to f_in, f_out): see Liquid3D::AHEAD
+  const void* fi[27];
+  void* fo[27];
 };
 
 // EXT: the extended model -- pairs' crystal axes turned about z (dAdq_pair)
@@ -314,7 +318,7 @@ __device__ __forceinline__ void general_tile(const DevParams<Real>& P, const Ste
       for (int a = 0; a < NP; ++a)
 #pragma unroll
         for (int b = a + 1; b < NP; ++b) {
-          if ((grp & ((1u << a) | (1u << b))) != ((1u << a) | (1u << b))) continue;
+          if ((NP == 2 || EXT) && (grp & ((1u << a) | (1u << b))) != ((1u << a) | (1u << b))) continue;
           const Real gv = P.gamma[a][b] * flux(a, b, pf[a] * gn[b] - pf[b] * gn[a], pf[a] * g1[b] - pf[b] * g1[a],
                                                pf[a] * g2[b] - pf[b] * g2[a]);
           fl[a] -= pf[b] * gv;
