@@ -322,11 +322,6 @@ __device__ __forceinline__ long long liquid_flag_index(int bx, int by, int v, in
   return ((long long)v * gy + by) * gx + bx;
 }
 
-// The reach of the z segment starting at plane z0 of xy tile (bx, by) -- the
-// 3 x 3 tiles around it (wrapped on periodic axes, skipped beyond walls,
-// where a wall mirrors the tile's own cells) on planes z0 - 2 .. z0 + ZS + 1
-// (folded like the cells) -- is flagged pure liquid.  Every thread of the CTA
-// calls it; the answer is uniform.
 // The flag of tile t (0 .. 8) of the 3 x 3 around (bx, by) in plane v (any
 // plane the reach names; set where the tile lies beyond a wall).
 template <class Real>
@@ -345,6 +340,11 @@ __device__ __forceinline__ bool liquid_flag_near(const DevParams<Real>& P, const
   return skip || flags[liquid_flag_index(c[0], c[1], fold_axis(P, v, 2), gx, gy)] != 0;
 }
 
+// The reach of the z segment starting at plane z0 of xy tile (bx, by) -- the
+// 3 x 3 tiles around it (wrapped on periodic axes, skipped beyond walls,
+// where a wall mirrors the tile's own cells) on planes z0 - 2 .. z0 + ZS + 1
+// (folded like the cells) -- is flagged pure liquid.  Every thread of the CTA
+// calls it; the answer is uniform.
 template <int ZS, class Real>
 __device__ __forceinline__ bool liquid_reach(const DevParams<Real>& P, const unsigned char* __restrict__ flags,
                                              int bx, int by, int z0, int gx, int gy) {
@@ -877,7 +877,7 @@ __device__ __forceinline__ Real composition(const DevParams<Real>& P, const Real
 // (3.2 GB read and written) take 466 us, 6.8 TB/s; one cell a thread with
 // each store after its load on two CTAs an SM, which this replaces, 949 us.
 template <int D, int Q, int NP, int NC, class Real, class Store, class Out, int V>
-__global__ void __launch_bounds__(256, 2)
+__global__ void __launch_bounds__(256, V == 1 ? 4 : 2)
     fields_kernel(const DevParams<Real> P, const Real* __restrict__ phi, const Real* __restrict__ mu_in,
                   const Store* __restrict__ f, const double* __restrict__ clock, Out* __restrict__ o_phi,
                   Out* __restrict__ o_mu, Out* __restrict__ o_c, Out* __restrict__ o_f, Out* __restrict__ o_rho,

@@ -67,9 +67,10 @@ struct Ops {
 };
 
 // Grid of the exchange kernels (state load, field write-back): a grid-stride
-// loop over `per_sm` CTAs of 256 threads per SM.  Two keep enough accesses in
-// flight for the host link and leave room on every SM for the other of the
-// two kernels, which may run at the same time on another stream; between
+// loop over `per_sm` CTAs of 256 threads per SM.  Two (of the field kernel's
+// 16-byte words, which take half an SM's registers a CTA, one) keep enough
+// accesses in flight for the host link and leave room on every SM for the other
+// of the two kernels, which may run at the same time on another stream; between
 // device buffers nothing runs beside them, and HBM wants more loads in
 // flight (1001^2 cells, one a thread: the load 21.5 us with two, 14.0 us with
 // eight).
@@ -253,7 +254,8 @@ struct Impl {
     // against 11.2 us with V = 2).
     const bool vec = P.n[0] % V == 0 && cells / V >= 152 * threads && al16(io.o_phi) && al16(io.o_mu) && al16(io.o_c) &&
                      al16(io.o_f) && al16(io.o_rho) && al16(io.o_u) && al16(io.o_dev);
-    const unsigned blocks = exchange_blocks(vec ? cells / V : cells, threads, io.link ? kLinkCtas : kDeviceCtas);
+    const unsigned blocks =
+        exchange_blocks(vec ? cells / V : cells, threads, !io.link ? kDeviceCtas : (vec ? kLinkCtas / 2 : kLinkCtas));
     auto go = [&](auto kernel) {
       kernel<<<blocks, threads, 0, s>>>(
           P, static_cast<const Real*>(io.phi), static_cast<const Real*>(io.mu), static_cast<const Store*>(io.f),

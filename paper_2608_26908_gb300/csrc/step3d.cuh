@@ -52,7 +52,7 @@ struct Step3D {
   // against 1.91 ms on the ternary eutectic); FP64 and 27 populations: one
   static constexpr int MIN_CTAS = (sizeof(Real) == 4 && QQ == 19) ? 2 : 1;
   // both paths in one launch where they have the same register budget and
-  // the general path's shared memory is small (two phases: 46 KB).  A launch
+  // the general path's shared memory is small (two phases: 37 KB).  A launch
   // reserves its largest path's shared memory for every CTA, and with more
   // phases (96 KB) the liquid tiles are left too little L1 for their loads
   // in flight: the ternary eutectic takes 1.88 ms a step in one launch,
@@ -155,9 +155,11 @@ __device__ __forceinline__ void general_tile(const DevParams<Real>& P, const Ste
       return P.ceq[a][i];
   };
   // Three and four phases: the plain kernels are for isotropic problems, and an
-  // anisotropic one takes the extended model's (the launcher's choice): with
-  // the anisotropic stencils in it the code outgrows the instruction cache
-  // (ncu: 4.0 of 14 stall cycles an issue wait for instructions, 0.4 without).
+  // anisotropic one takes the extended model's (the launcher's choice).  The
+  // code of a plane is larger than the instruction cache, and the waits for
+  // instructions are the general path's first stall; with the anisotropic
+  // stencils in it the eutectic 150 x 130 x 171 half solid takes 481 us of
+  // general path a step, without them 436.
   const bool aniso = (NP == 2 || EXT) && P.aniso != 0;
   const bool has_walls = (P.wall[0] | P.wall[1] | P.wall[2]) != 0;  // obstacle rows
   // vertical index of a plane the kernel reads: folded on the whole grid
@@ -251,9 +253,9 @@ __device__ __forceinline__ void general_tile(const DevParams<Real>& P, const Ste
   // ia) and its neighbour B along axis d: the d-th component of -sum_{b != a}
   // gamma_ab phi_b dA/dq(q_ab) for every phase.  Two phases: q_01 = grad phi_1
   // on the face (phi_0 + phi_1 = 1) and the update needs gamma dA/dq, the
-  // difference of the two fluxes, alone: V = dA/dq.  d is a run-time value so
-  // that the code is there once: with a copy a face the general path waits for
-  // its instructions (ncu: 2.4 of 14 stall cycles an issue).
+  // difference of the two fluxes, alone: V = dA/dq.  (Callers unroll over d: one
+  // copy of the code with d at run time ends the waits for instructions, but
+  // executes a quarter more of them, 419 against 396 us on the grown eutectic.)
   constexpr int NF = S::NF;
   auto pf_face = [&](int pa, int ia, int d, bool closed, Real* fl) {
 #pragma unroll
@@ -713,8 +715,7 @@ __device__ __forceinline__ void general_tile(const DevParams<Real>& P, const Ste
       const int fzm = vz(M);
       const bool walls = has_walls;
       // d = 2: the z-face (M, M+1) of this column, for the carry; then, on the
-      // planes it updates, the +x and +y faces into shared memory (one copy of
-      // the code, as for the phase field)
+      // planes it updates, the +x and +y faces into shared memory
 #pragma unroll
       for (int f = 0; f < 3; ++f) {
         if (f > 0 && M == z0 - 1) continue;

@@ -43,9 +43,10 @@ struct Liquid3D {
   static constexpr size_t bytes = sizeof(Real) * 2 * 2 * NC * NT;
   // Two phases with FP32 populations: a plane's loads are issued before the
   // barrier of the plane below, from a pointer a population (dendrite 256^3:
-  // 666 us a step against 673; four phases 1655 against 1651, and 16-bit
-  // populations, which then pay for packing them, 733 against 603).
-  static constexpr bool AHEAD = NP == 2 && sizeof(Store) == 4 && sizeof(Real) == 4;
+  // 666 us a step against 673; not four phases, 1655 against 1651, nor 16-bit
+  // populations, which then pay for packing them, 733 against 603, nor D3Q27,
+  // 120^3: 206 against 191).
+  static constexpr bool AHEAD = NP == 2 && QQ == 19 && sizeof(Store) == 4 && sizeof(Real) == 4;
 };
 
 // The liquid path for n planes from z0 of xy tile (bx, by) (z0 + n <= v_hi).
