@@ -67,9 +67,8 @@ struct Ops {
 };
 
 // Grid of the exchange kernels (state load, field write-back): a grid-stride
-// loop over `per_sm` CTAs of 256 threads per SM.  Two (of the field kernel's
-// 16-byte words, which take half an SM's registers a CTA, one) keep enough
-// accesses in flight for the host link and leave room on every SM for the other
+// loop over `per_sm` CTAs of 256 threads per SM.  Two keep enough accesses in
+// flight for the host link and leave room on every SM for the other
 // of the two kernels, which may run at the same time on another stream; between
 // device buffers nothing runs beside them, and HBM wants more loads in
 // flight (1001^2 cells, one a thread: the load 21.5 us with two, 14.0 us with
@@ -122,6 +121,7 @@ struct Impl {
   using S3 = Step3D<NP, NC, Real, Store, (D == 3 ? Q : 19)>;
   using SL = Liquid3D<NP, NC, Real, Store, (D == 3 ? Q : 19), EXT>;
   // 3D: dynamic shared memory of step3d_kernel (both paths when it runs both)
+  static constexpr size_t shrink3d_bytes = Step3D<NP, NC, Real, Store, (D == 3 ? Q : 19), true>::bytes;
   static constexpr size_t step3d_bytes = !S3::ONE_LAUNCH ? S3::bytes : (S3::bytes > SL::bytes ? S3::bytes : SL::bytes);
 
   static cudaError_t configure() {
@@ -139,7 +139,7 @@ struct Impl {
                                cudaFuncAttributeMaxDynamicSharedMemorySize, (int)step3d_bytes);
       if (e == cudaSuccess)
         e = cudaFuncSetAttribute(step3d_kernel<NP, NC, Real, Store, true, Q, EXT>,
-                                 cudaFuncAttributeMaxDynamicSharedMemorySize, (int)step3d_bytes);
+                                 cudaFuncAttributeMaxDynamicSharedMemorySize, (int)shrink3d_bytes);
       if constexpr (!S3::ONE_LAUNCH) {
         if (e == cudaSuccess)
           e = cudaFuncSetAttribute(step3d_liquid_kernel<NP, NC, Real, Store, Q, EXT>,
@@ -184,7 +184,7 @@ struct Impl {
         sio.fo[k] = static_cast<char*>(io.f_out) + P.f_to[k];
       }
       if (P.shrink)
-        step3d_kernel<NP, NC, Real, Store, true, Q, EXT><<<grid, S3::NT, step3d_bytes, s>>>(P, sio);
+        step3d_kernel<NP, NC, Real, Store, true, Q, EXT><<<grid, S3::NT, shrink3d_bytes, s>>>(P, sio);
       else
         step3d_kernel<NP, NC, Real, Store, false, Q, EXT><<<grid, S3::NT, step3d_bytes, s>>>(P, sio);
       // the tiles whose reach is pure liquid (step3d_kernel returned there)
@@ -252,10 +252,12 @@ struct Impl {
     // A grid too small to give every SM a CTA of V cells a thread is bound by a
     // thread's own chain, and takes one cell a thread (FP64 128^2: 7.5 us
     // against 11.2 us with V = 2).
-    const bool vec = P.n[0] % V == 0 && cells / V >= 152 * threads && al16(io.o_phi) && al16(io.o_mu) && al16(io.o_c) &&
+    // Over the host link the words gain nothing, and their registers leave the
+    // load beside the write-back too little of an SM (two CTAs an SM: eutectic3d
+    // end to end 1.82k -> 1.56k MLUPS; one: eutectic2d 3.31k -> 3.24k).
+    const bool vec = !io.link && P.n[0] % V == 0 && cells / V >= 152 * threads && al16(io.o_phi) && al16(io.o_mu) && al16(io.o_c) &&
                      al16(io.o_f) && al16(io.o_rho) && al16(io.o_u) && al16(io.o_dev);
-    const unsigned blocks =
-        exchange_blocks(vec ? cells / V : cells, threads, !io.link ? kDeviceCtas : (vec ? kLinkCtas / 2 : kLinkCtas));
+    const unsigned blocks = exchange_blocks(vec ? cells / V : cells, threads, io.link ? kLinkCtas : kDeviceCtas);
     auto go = [&](auto kernel) {
       kernel<<<blocks, threads, 0, s>>>(
           P, static_cast<const Real*>(io.phi), static_cast<const Real*>(io.mu), static_cast<const Store*>(io.f),

@@ -38,14 +38,14 @@ struct Block3D {
   static constexpr int BX = 32, BY = 16, ZS = sizeof(Real) == 4 ? 6 : 16;
 };
 
-template <int NP, int NC, class Real, class Store, int QQ = 19>
+template <int NP, int NC, class Real, class Store, int QQ = 19, bool SHRINK = false>
 struct Step3D {
   static constexpr int BX = Block3D<Real>::BX, BY = Block3D<Real>::BY, ZS = Block3D<Real>::ZS;
   static constexpr int NT = BX * BY, Q = QQ;  // D3Q19 or D3Q27
   static constexpr int NS = PhiStore<NP>::NS;
   // values of a phase-field face: two phases need the difference of their two
-  // fluxes alone (see pf_face)
-  static constexpr int NF = NP == 2 ? 1 : NP;
+  // fluxes alone (see pf_face; with shrinkage both, see pf_flux)
+  static constexpr int NF = NP == 2 && !SHRINK ? 1 : NP;
   // resident CTAs per SM the register budget is cut for: two (64 registers)
   // on D3Q19 in FP32, for any number of phases (three and four phases spill
   // a few dozen bytes, yet two CTAs of 64 registers beat one of 128: 1.79
@@ -105,7 +105,7 @@ struct Step3DIO {
 template <int NP, int NC, class Real, class Store, bool SHRINK, int QQ, bool EXT>
 __device__ __forceinline__ void general_tile(const DevParams<Real>& P, const Step3DIO& io, int bx, int by, int bz,
                                              int gxt, int gyt) {
-  using S = Step3D<NP, NC, Real, Store, QQ>;
+  using S = Step3D<NP, NC, Real, Store, QQ, SHRINK>;
   using Lat = Lattice<QQ>;
   constexpr int BX = S::BX, BY = S::BY, ZS = S::ZS, NT = S::NT, Q = QQ;
   constexpr int W2 = S::W2, H2 = S::H2, C2 = S::C2, NS = S::NS;
@@ -160,7 +160,7 @@ __device__ __forceinline__ void general_tile(const DevParams<Real>& P, const Ste
   // instructions are the general path's first stall; with the anisotropic
   // stencils in it the eutectic 150 x 130 x 171 half solid takes 481 us of
   // general path a step, without them 436.
-  const bool aniso = (NP == 2 || EXT) && P.aniso != 0;
+  const bool aniso = (NP == 2 || EXT || SHRINK) && P.aniso != 0;
   const bool has_walls = (P.wall[0] | P.wall[1] | P.wall[2]) != 0;  // obstacle rows
   // vertical index of a plane the kernel reads: folded on the whole grid
   // (walls mirror, periodic wraps), then kept inside the planes the buffers
@@ -329,6 +329,63 @@ __device__ __forceinline__ void general_tile(const DevParams<Real>& P, const Ste
     }
   };
 
+  // With shrinkage the force is the difference of phi^{n+1} and phi^n, some 1e-4
+  // of either: another rounding of the update is a thousand times larger in the
+  // force, and flips the stored rounding of 16-bit populations.  So this variant
+  // evaluates the fluxes phase by phase, in the order of the definition (A and B
+  // are cells ia, ib of planes pa, pb).
+  auto pf_flux = [&](int pa, int ia, int pb, int ib, int d, bool closed, Real* fl) {
+#pragma unroll
+    for (int a = 0; a < NP; ++a) fl[a] = Real(0);
+    // the cells the stencil reads
+    unsigned grp;
+    Real pf[NP], g3[NP][3];
+    if (d == 2) {
+      grp = MK(pa, ia) | MK(pb, ib) | MK(pa, ia + 1) | MK(pb, ib + 1) | MK(pa, ia - 1) |
+            MK(pb, ib - 1) | MK(pa, ia + W2) | MK(pb, ib + W2) | MK(pa, ia - W2) | MK(pb, ib - W2);
+    } else {
+      const int st = d == 0 ? W2 : 1;
+      grp = MK(pa, ia) | MK(pb, ib) | MK(pa, ia + st) | MK(pb, ib + st) | MK(pa, ia - st) |
+            MK(pb, ib - st) | MK(pa - 1, ia) | MK(pb - 1, ib) | MK(pa + 1, ia) | MK(pb + 1, ib);
+    }
+    if (__popc(grp) < 2 || closed) return;
+    // A phase whose mask bit is clear in every cell the stencil reads is
+    // exactly 0 there: its face value and gradient are 0, so every pair it
+    // belongs to has q = 0 and contributes exactly 0.  Such phases and pairs
+    // are skipped (two or three of the four phases at most interfaces).
+#pragma unroll
+    for (int a = 0; a < NP; ++a) {
+      pf[a] = Real(0);
+      g3[a][0] = g3[a][1] = g3[a][2] = Real(0);
+      if (!(grp & (1u << a))) continue;
+      const Real va = PH(pa, a, ia), vb = PH(pb, a, ib);
+      pf[a] = Real(0.5) * (va + vb);
+      g3[a][d] = vb - va;
+      if (!P.aniso) continue;  // dA/dq = 2 q: only q_d enters the flux
+      if (d == 2) {
+        g3[a][0] = Real(0.25) * (PH(pa, a, ia + 1) + PH(pb, a, ib + 1) - PH(pa, a, ia - 1) - PH(pb, a, ib - 1));
+        g3[a][1] = Real(0.25) * (PH(pa, a, ia + W2) + PH(pb, a, ib + W2) - PH(pa, a, ia - W2) - PH(pb, a, ib - W2));
+      } else {
+        const int st = d == 0 ? W2 : 1;  // the other in-plane axis
+        g3[a][1 - d] = Real(0.25) * (PH(pa, a, ia + st) + PH(pb, a, ib + st) - PH(pa, a, ia - st) - PH(pb, a, ib - st));
+        g3[a][2] = Real(0.25) * (PH(pa + 1, a, ia) + PH(pb + 1, a, ib) - PH(pa - 1, a, ia) - PH(pb - 1, a, ib));
+      }
+    }
+#pragma unroll
+    for (int a = 0; a < NP; ++a)
+#pragma unroll
+      for (int b = a + 1; b < NP; ++b) {
+        const Real gab = P.gamma[a][b];
+        if (gab == Real(0) || (grp & ((1u << a) | (1u << b))) != ((1u << a) | (1u << b))) continue;
+        Real q[3];
+#pragma unroll
+        for (int t = 0; t < 3; ++t) q[t] = pf[a] * g3[b][t] - pf[b] * g3[a][t];
+        const Real v = dAdq_pair<3, EXT>(P, a, b, q, d);
+        fl[a] -= gab * pf[b] * v;
+        fl[b] += gab * pf[a] * v;
+      }
+  };
+
   const int L0 = z0 - 2, L1 = z0 + ZS + 1;
   for (int L = L0; L <= L1; ++L) {
     const int C = L - 1, M = L - 2;
@@ -461,7 +518,39 @@ __device__ __forceinline__ void general_tile(const DevParams<Real>& P, const Ste
 #pragma unroll
       for (int a = 0; a < NF; ++a) pfz_hi[a] = Real(0);
     } else {
+      if constexpr (SHRINK) {
       if (pfC) {
+        // in-plane faces of plane C into shared memory
+        Real fl[NP];
+        const bool cx_hi = P.bc[0] == kWall && (gx + 1 == 0 || gx + 1 == nx);
+        pf_flux(C, r2, C, r2 + 1, 0, cx_hi, fl);
+#pragma unroll
+        for (int a = 0; a < NP; ++a) s_flux[a * (S::PFX + S::PFY) + ty * (BX + 1) + tx + 1] = fl[a];
+        if (tx == 0) {
+          const bool cx_lo = P.bc[0] == kWall && (gx == 0 || gx == nx);
+          pf_flux(C, r2 - 1, C, r2, 0, cx_lo, fl);
+#pragma unroll
+          for (int a = 0; a < NP; ++a) s_flux[a * (S::PFX + S::PFY) + ty * (BX + 1)] = fl[a];
+        }
+        const bool cy_hi = P.bc[1] == kWall && (gy + 1 == 0 || gy + 1 == ny);
+        pf_flux(C, r2, C, r2 + W2, 1, cy_hi, fl);
+#pragma unroll
+        for (int a = 0; a < NP; ++a) s_flux[a * (S::PFX + S::PFY) + S::PFX + (ty + 1) * BX + tx] = fl[a];
+        if (ty == 0) {
+          const bool cy_lo = P.bc[1] == kWall && (gy == 0 || gy == ny);
+          pf_flux(C, r2 - W2, C, r2, 1, cy_lo, fl);
+#pragma unroll
+          for (int a = 0; a < NP; ++a) s_flux[a * (S::PFX + S::PFY) + S::PFX + tx] = fl[a];
+        }
+        // z-faces of this column: (C, C+1), and (C-1, C) on the first plane
+        const bool cz_hi = P.bc[2] == kWall && (C + 1 == 0 || C + 1 == nz);
+        pf_flux(C, r2, C + 1, r2, 2, cz_hi, pfz_hi);
+        if (C == z0 - 1) {
+          const bool cz_lo = P.bc[2] == kWall && (C == 0 || C == nz);
+          pf_flux(C - 1, r2, C, r2, 2, cz_lo, pfz_lo);
+        }
+      }
+      } else if (pfC) {
         // f = 0: the first face of every row and column, by the lanes of two
         // warps; 1, 2: the +x and +y faces into shared memory; 3: the z-face
         // (C, C+1); 4, on the first plane: (C-1, C)
@@ -516,7 +605,85 @@ __device__ __forceinline__ void general_tile(const DevParams<Real>& P, const Ste
         Real mu[NC];
 #pragma unroll
         for (int i = 0; i < NC; ++i) mu[i] = s_mu[(slot2(C) * NC + i) * NT + tid];
-        if constexpr (NP == 2) {
+        if constexpr (SHRINK) {  // in the order of the definition, see pf_flux
+          Real div[NP], gc[NP][3];
+#pragma unroll
+          for (int a = 0; a < NP; ++a) {
+            const Real* fa = s_flux + a * (S::PFX + S::PFY);
+            div[a] = (fa[ty * (BX + 1) + tx + 1] - fa[ty * (BX + 1) + tx]) +
+                     (fa[S::PFX + (ty + 1) * BX + tx] - fa[S::PFX + ty * BX + tx]) + (pfz_hi[a] - pfz_lo[a]);
+            // a phase absent from the 3x3x3 neighbourhood has a zero central
+            // gradient, and its pairs contribute exactly 0 below
+            gc[a][0] = gc[a][1] = gc[a][2] = Real(0);
+            if (!(act & (1u << a))) continue;
+            gc[a][0] = Real(0.5) * (PH(C, a, r2 + 1) - PH(C, a, r2 - 1));
+            gc[a][1] = Real(0.5) * (PH(C, a, r2 + W2) - PH(C, a, r2 - W2));
+            gc[a][2] = Real(0.5) * (PH(C + 1, a, r2) - PH(C - 1, a, r2));
+          }
+          Real ph[NP];
+#pragma unroll
+          for (int a = 0; a < NP; ++a) ph[a] = out[a];
+          Real dadphi[NP];
+#pragma unroll
+          for (int a = 0; a < NP; ++a) dadphi[a] = Real(0);
+#pragma unroll
+          for (int a = 0; a < NP; ++a)
+#pragma unroll
+            for (int b = a + 1; b < NP; ++b) {
+              const Real gab = P.gamma[a][b];
+              if (gab == Real(0) || (act & ((1u << a) | (1u << b))) != ((1u << a) | (1u << b))) continue;
+              Real q[3], v[3];
+#pragma unroll
+              for (int t = 0; t < 3; ++t) q[t] = ph[a] * gc[b][t] - ph[b] * gc[a][t];
+              dAdq_vec_pair<3, EXT>(P, a, b, q, v);
+              dadphi[a] += gab * (v[0] * gc[b][0] + v[1] * gc[b][1] + v[2] * gc[b][2]);
+              dadphi[b] -= gab * (v[0] * gc[a][0] + v[1] * gc[a][1] + v[2] * gc[a][2]);
+            }
+          Real psi[NP];
+#pragma unroll
+          for (int b = 0; b < NP; ++b) {
+            Real sv = P.S[b] * theta;
+#pragma unroll
+            for (int i = 0; i < NC; ++i) sv -= mu[i] * mu[i] * P.inv4A[b] + mu[i] * ceq_of(b, i, fzC);
+            psi[b] = sv;
+          }
+          Real rate[NP];
+#pragma unroll
+          for (int a = 0; a < NP; ++a) {
+            Real obst = Real(0), drv = Real(0);
+#pragma unroll
+            for (int b = 0; b < NP; ++b) {
+              if (b != a) obst += P.gamma[a][b] * ph[b];
+              drv += psi[b] * interp_dh<NP>(ph, b, a);
+            }
+            rate[a] = P.eps * (div[a] - dadphi[a]) - P.obst * obst - drv;
+          }
+          int na = 0;
+          Real lam = Real(0);
+#pragma unroll
+          for (int a = 0; a < NP; ++a)
+            if (act & (1u << a)) {
+              lam += rate[a];
+              ++na;
+            }
+          lam = lam / Real(na);
+          Real uv[NP];
+          int m = 0;
+#pragma unroll
+          for (int a = 0; a < NP; ++a)
+            if (act & (1u << a)) uv[m++] = ph[a] + P.mob_eps * (rate[a] - lam);
+          if (NP == 2) {
+            Real sv = uv[1];
+            sv = sv < Real(0) ? Real(0) : (sv > Real(1) ? Real(1) : sv);
+            out[1] = sv;
+            out[0] = Real(1) - sv;
+          } else {
+            project_simplex<Real, NP>(uv, m);
+            m = 0;
+#pragma unroll
+            for (int a = 0; a < NP; ++a) out[a] = (act & (1u << a)) ? uv[m++] : Real(0);
+          }
+        } else if constexpr (NP == 2) {
           // Lambda is the mean of the two rates, so phi_1 moves by half their
           // difference; the centre terms da/dphi are equal and cancel, and
           // dh_1/dphi_1 = dh_0/dphi_0 = 6 s (1 - s)

@@ -301,7 +301,7 @@ __device__ __forceinline__ void liquid_tiles(const DevParams<Real>& P, const Ste
 template <int NP, int NC, class Real, class Store, bool SHRINK = false, int QQ = 19, bool EXT = false>
 __global__ void __launch_bounds__(Step3D<NP, NC, Real, Store, QQ>::NT, Step3D<NP, NC, Real, Store, QQ>::MIN_CTAS)
     step3d_kernel(const DevParams<Real> P, const Step3DIO io) {
-  using S = Step3D<NP, NC, Real, Store, QQ>;
+  using S = Step3D<NP, NC, Real, Store, QQ, SHRINK>;
   constexpr int ZS = S::ZS;
   const int gxt = gridDim.x, gyt = gridDim.y, gzt = (P.v_hi - P.v_lo + ZS - 1) / ZS;
   const int bx = blockIdx.x, by = blockIdx.y;
