@@ -121,7 +121,7 @@ struct Impl {
   using S3 = Step3D<NP, NC, Real, Store, (D == 3 ? Q : 19)>;
   using SL = Liquid3D<NP, NC, Real, Store, (D == 3 ? Q : 19), EXT>;
   // 3D: dynamic shared memory of step3d_kernel (both paths when it runs both)
-  static constexpr size_t shrink3d_bytes = Step3D<NP, NC, Real, Store, (D == 3 ? Q : 19), true>::bytes;
+  using SS = Step3D<NP, NC, Real, Store, (D == 3 ? Q : 19), true>;
   static constexpr size_t step3d_bytes = !S3::ONE_LAUNCH ? S3::bytes : (S3::bytes > SL::bytes ? S3::bytes : SL::bytes);
 
   static cudaError_t configure() {
@@ -139,7 +139,7 @@ struct Impl {
                                cudaFuncAttributeMaxDynamicSharedMemorySize, (int)step3d_bytes);
       if (e == cudaSuccess)
         e = cudaFuncSetAttribute(step3d_kernel<NP, NC, Real, Store, true, Q, EXT>,
-                                 cudaFuncAttributeMaxDynamicSharedMemorySize, (int)shrink3d_bytes);
+                                 cudaFuncAttributeMaxDynamicSharedMemorySize, (int)SS::bytes);
       if constexpr (!S3::ONE_LAUNCH) {
         if (e == cudaSuccess)
           e = cudaFuncSetAttribute(step3d_liquid_kernel<NP, NC, Real, Store, Q, EXT>,
@@ -183,8 +183,9 @@ struct Impl {
         sio.fi[k] = static_cast<const char*>(io.f_in) + P.f_at[k];
         sio.fo[k] = static_cast<char*>(io.f_out) + P.f_to[k];
       }
-      if (P.shrink)
-        step3d_kernel<NP, NC, Real, Store, true, Q, EXT><<<grid, S3::NT, shrink3d_bytes, s>>>(P, sio);
+      if (P.shrink)  // (no liquid dispatch: every tile takes the general path)
+        step3d_kernel<NP, NC, Real, Store, true, Q, EXT>
+            <<<dim3((P.n[0] + SS::OX - 1) / SS::OX, (P.n[1] + SS::OY - 1) / SS::OY, gz), SS::NT, SS::bytes, s>>>(P, sio);
       else
         step3d_kernel<NP, NC, Real, Store, false, Q, EXT><<<grid, S3::NT, step3d_bytes, s>>>(P, sio);
       // the tiles whose reach is pure liquid (step3d_kernel returned there)

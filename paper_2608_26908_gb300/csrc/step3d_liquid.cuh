@@ -299,7 +299,7 @@ __device__ __forceinline__ void liquid_tiles(const DevParams<Real>& P, const Ste
 // shared memory, see ONE_LAUNCH) step3d_kernel takes the general tiles and
 // step3d_liquid_kernel, launched after it, the others.
 template <int NP, int NC, class Real, class Store, bool SHRINK = false, int QQ = 19, bool EXT = false>
-__global__ void __launch_bounds__(Step3D<NP, NC, Real, Store, QQ>::NT, Step3D<NP, NC, Real, Store, QQ>::MIN_CTAS)
+__global__ void __launch_bounds__(Step3D<NP, NC, Real, Store, QQ, SHRINK>::NT, Step3D<NP, NC, Real, Store, QQ>::MIN_CTAS)
     step3d_kernel(const DevParams<Real> P, const Step3DIO io) {
   using S = Step3D<NP, NC, Real, Store, QQ, SHRINK>;
   constexpr int ZS = S::ZS;
