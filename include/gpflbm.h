@@ -193,7 +193,9 @@ gpflbm_status gpflbm_halo_bytes(gpflbm_t h, size_t* bytes);
 gpflbm_status gpflbm_halo_pack(gpflbm_t h, int side, void* msg, void* stream);
 gpflbm_status gpflbm_halo_unpack(gpflbm_t h, int side, const void* msg, void* stream);
 
-/* Replace the model parameters (same grid, phase and solute counts). */
+/* Replace the model parameters (same grid, phase and solute counts).  Host
+ * work only: steps queued before the call keep the parameters they were queued
+ * with, and need not have finished. */
 gpflbm_status gpflbm_set_params(gpflbm_t h, const gpflbm_params* params);
 
 /* Flags of the src_is_device / dst_is_device arguments of gpflbm_set_state

@@ -49,6 +49,7 @@ struct gpflbm_s {
   int cur;            // buffer holding the current state
   long long t;        // step counter of the current state
   bool has_state;
+  bool flags_stale;   // the liquid flags of both buffers await the next step (set_params)
   cudaStream_t capture;
   // adjoint: the stream that recomputes segments, and its events
   cudaStream_t aux;
@@ -493,6 +494,21 @@ cudaError_t classify(gpflbm_t h, int buf, cudaStream_t s) {
                           static_cast<unsigned char*>(at(h, h->lay.flags[buf])), s);
 }
 
+// Before a step on stream s: the flags that set_params left stale, of both
+// buffers (the liquid path also reads those of the buffer it writes).  Here
+// rather than in set_params, which has no stream: what still writes the
+// buffers is ordered before the caller's next step, on that step's stream.  A
+// step that is being captured takes the classification into the graph, which
+// may never run: the flags stay stale for the steps that are not.
+cudaError_t refresh_flags(gpflbm_t h, cudaStream_t s) {
+  if (!h->flags_stale || !h->pf.liq_dispatch) return cudaSuccess;
+  cudaStreamCaptureStatus c = cudaStreamCaptureStatusNone;
+  cudaError_t e = cudaStreamIsCapturing(s, &c);
+  for (int i = 0; i < 2 && e == cudaSuccess; ++i) e = classify(h, i, s);
+  if (e == cudaSuccess && c == cudaStreamCaptureStatusNone) h->flags_stale = false;
+  return e;
+}
+
 // A slab steps only with both halos next to a neighbouring slab written
 // since its last step; the step then uses them up.
 gpflbm_status slab_ready(gpflbm_t h, const char* what) {
@@ -715,14 +731,8 @@ gpflbm_status gpflbm_set_params(gpflbm_t h, const gpflbm_params* params) {
   set_device_params(h);
   drop_graphs(h);  // parameters are baked into captured launches
   ++h->mut;
-  if (h->has_state && h->pf.liq_dispatch && !had) {
-    // the flags were not kept while every tile took the general path (the
-    // liquid path also reads those of the buffer it writes)
-    cudaError_t e = classify(h, h->cur, nullptr);
-    if (e == cudaSuccess) e = classify(h, 1 - h->cur, nullptr);
-    if (e == cudaSuccess) e = cudaStreamSynchronize(nullptr);
-    if (e != cudaSuccess) return cuda_fail(h, e, "set_params: liquid tiles");
-  }
+  // the flags were not kept while every tile took the general path
+  if (h->has_state && h->pf.liq_dispatch && !had) h->flags_stale = true;
   return GPFLBM_OK;
 }
 
@@ -848,6 +858,10 @@ gpflbm_status gpflbm_step(gpflbm_t h, int n_steps, void* stream) {
   }
   cudaStream_t s = static_cast<cudaStream_t>(stream);
   ++h->mut;
+  if (n_steps > 0) {
+    cudaError_t e = refresh_flags(h, s);
+    if (e != cudaSuccess) return cuda_fail(h, e, "step: liquid tiles");
+  }
   int left = n_steps;
   while (left > 0) {
     cudaError_t e;
@@ -942,7 +956,9 @@ gpflbm_status gpflbm_step_timed(gpflbm_t h, void* const* events, void* stream) {
   cudaStream_t s = static_cast<cudaStream_t>(stream);
   ++h->mut;
   const gpflbm::StepIO io = step_io(h, h->cur);
-  cudaError_t e = cudaEventRecord(static_cast<cudaEvent_t>(events[0]), s);
+  cudaError_t e = refresh_flags(h, s);
+  if (e != cudaSuccess) return cuda_fail(h, e, "step_timed: liquid tiles");
+  e = cudaEventRecord(static_cast<cudaEvent_t>(events[0]), s);
   if (e == cudaSuccess) e = stepper(h)->step(dev_params(h), io, s);
   if (e == cudaSuccess) e = cudaEventRecord(static_cast<cudaEvent_t>(events[1]), s);
   if (e != cudaSuccess) return cuda_fail(h, e, "step_timed");

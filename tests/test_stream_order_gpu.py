@@ -1,0 +1,44 @@
+"""Calls on a stream that does not synchronise with the legacy default stream:
+what one call queues is finished before the next one, without a wait between
+them, reads or rewrites it."""
+import copy
+
+import numpy as np
+import pytest
+
+from paper_2608_26908_gb300 import gpflbm, inputs
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.mark.parametrize("name", ["dendrite3d", "eutectic3d"])
+def test_parameters_changed_with_steps_in_flight(name):
+    """Shrinkage off again while shrinkage steps run: the liquid flags of both
+    buffers are taken after those steps, so the steps that follow are those of
+    a run that waits before the change."""
+    import torch
+
+    sc = inputs.scenario(name, nx=120, ny=112, nz=100)
+    sc["init"]["height" if name == "eutectic3d" else "radius"] = 30
+    shrink = copy.deepcopy(sc)
+    shrink["params"]["eta_rho"][1] = 0.1
+    state = [torch.as_tensor(a, dtype=torch.float32, device="cuda") for a in inputs.initial_state(sc)]
+    torch.cuda.synchronize()
+
+    def run(wait):
+        side = torch.cuda.Stream()
+        with torch.cuda.stream(side):
+            sim = gpflbm.Sim(sc)
+            sim.set_state(*state)
+            sim.step(3)
+            sim.set_params(shrink)
+            sim.step(41)
+            if wait:
+                torch.cuda.synchronize()
+            sim.set_params(sc)
+            sim.step(5)
+            return sim.fields(("phi", "mu", "f"))
+
+    want, got = run(True), run(False)
+    for k in want:
+        np.testing.assert_array_equal(got[k], want[k], err_msg=k)
