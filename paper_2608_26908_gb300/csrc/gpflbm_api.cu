@@ -674,7 +674,13 @@ gpflbm_status create_impl(const gpflbm_grid* grid, int n_phases, int n_component
     delete h;
     return GPFLBM_ERR_CUDA;
   }
-  e = cudaMemset(h->ws, 0, h->lay.total);  // padding cells stay finite
+  // Padding cells stay finite, and no tile is flagged liquid.  The memset runs
+  // on the legacy default stream, which non-blocking streams do not wait for
+  // and which does not wait for them: earlier work on the caller's workspace
+  // is let finish first, and the memset before the caller's first load.
+  e = cudaDeviceSynchronize();
+  if (e == cudaSuccess) e = cudaMemset(h->ws, 0, h->lay.total);
+  if (e == cudaSuccess) e = cudaStreamSynchronize(nullptr);
   if (e != cudaSuccess) {
     std::fprintf(stderr, "gpflbm_create: %s\n", cudaGetErrorString(e));
     gpflbm_destroy(h);

@@ -42,3 +42,21 @@ def test_parameters_changed_with_steps_in_flight(name):
     want, got = run(True), run(False)
     for k in want:
         np.testing.assert_array_equal(got[k], want[k], err_msg=k)
+
+
+def test_a_state_loaded_right_after_creation_stays():
+    """The workspace is cleared before gpflbm_create returns: a load on a side
+    stream directly after it is not wiped."""
+    import torch
+
+    sc = inputs.scenario("eutectic3d", nx=256, ny=256, nz=128)
+    phi, mu = (torch.as_tensor(a, dtype=torch.float32, device="cuda") for a in inputs.initial_state(sc))
+    torch.cuda.synchronize()
+    side = torch.cuda.Stream()
+    with torch.cuda.stream(side):
+        sim = gpflbm.Sim(sc)
+        sim.set_state(phi, mu)
+        got = sim.fields(("phi", "mu"), device=True)
+        side.synchronize()
+        assert torch.equal(got["phi"].reshape(-1), phi.reshape(-1))
+        assert torch.equal(got["mu"].reshape(-1), mu.reshape(-1))
