@@ -1593,6 +1593,18 @@ gpflbm_status adjoint_run(gpflbm_t h, const gpflbm_objective* obj, int H, const 
   return GPFLBM_OK;
 }
 
+// A sweep that failed half-way may have left steps queued on the auxiliary
+// stream, which `s` does not wait for yet, and the workspace is not the
+// library's: it may be freed, or given to other work on `s`, as soon as the
+// call returns.
+gpflbm_status adjoint_finish(gpflbm_t h, gpflbm_status st, cudaStream_t s) {
+  if (st != GPFLBM_OK) {
+    cudaStreamSynchronize(s);
+    if (h->aux) cudaStreamSynchronize(h->aux);
+  }
+  return st;
+}
+
 }  // namespace
 
 extern "C" {
@@ -1637,7 +1649,7 @@ gpflbm_status gpflbm_adjoint(gpflbm_t h, const gpflbm_objective* obj, int horizo
     ws = static_cast<unsigned char*>(p);
     own = true;
   }
-  st = adjoint_run(h, obj, horizon, L, ws, J, dparams, dmu0, dst_is_device, s);
+  st = adjoint_finish(h, adjoint_run(h, obj, horizon, L, ws, J, dparams, dmu0, dst_is_device, s), s);
   if (own) {
     cudaStreamSynchronize(s);  // nothing may still use the block
     cudaFree(ws);
@@ -1672,7 +1684,7 @@ gpflbm_status gpflbm_vjp(gpflbm_t h, int horizon, int ckpt_every, void* workspac
     ws = static_cast<unsigned char*>(p);
     own = true;
   }
-  st = adjoint_run(h, nullptr, horizon, L, ws, nullptr, dparams, nullptr, flags, s, seed, grad);
+  st = adjoint_finish(h, adjoint_run(h, nullptr, horizon, L, ws, nullptr, dparams, nullptr, flags, s, seed, grad), s);
   if (own) {
     cudaStreamSynchronize(s);
     cudaFree(ws);
