@@ -354,14 +354,16 @@ class Sim:
         """A workspace from torch's caching allocator, used on the current
         stream, or None (the library allocates its own): a cudaMalloc and a
         cudaFree of gigabytes in every call take as long as 40 adjoint steps of
-        512 x 512 cells."""
+        512 x 512 cells.  The block stays in torch's cache after the call, for
+        the next one, until torch.cuda.empty_cache() or until torch itself runs
+        short; a cudaMalloc outside torch cannot have it back."""
         torch = self.torch
         n = ctypes.c_size_t()
         if lib().gpflbm_adjoint_workspace_bytes(self.h, int(horizon), int(ckpt_every), ctypes.byref(n)) != OK:
             return None
         try:
             return torch.empty(n.value, dtype=torch.uint8, device="cuda")
-        except torch.cuda.OutOfMemoryError:
+        except (torch.cuda.OutOfMemoryError, TypeError):  # TypeError: 2^63 bytes and more
             return None
 
     def adjoint(self, obj, horizon, ckpt_every, device=False, workspace=None):
@@ -403,7 +405,14 @@ class Sim:
         seed = np.ascontiguousarray(seed, dtype=self.dtype).reshape(11, self.cells)
         grad = np.empty((11, self.cells), dtype=self.dtype)
         dpar = (ctypes.c_double * 3)()
-        self._check(lib().gpflbm_vjp(self.h, int(horizon), int(ckpt_every), None, 0,
+        # from the same cache as adjoint()'s, which an allocation of the
+        # library's own could not use
+        workspace = self._adjoint_workspace(horizon, ckpt_every)
+        if workspace is not None:
+            wptr, wbytes = ctypes.c_void_p(workspace.data_ptr()), workspace.numel()
+        else:
+            wptr, wbytes = None, 0
+        self._check(lib().gpflbm_vjp(self.h, int(horizon), int(ckpt_every), wptr, wbytes,
                                      ctypes.c_void_p(seed.ctypes.data), ctypes.c_void_p(grad.ctypes.data),
                                      dpar, 0, _stream(self.torch)), "vjp")
         return grad, np.array(dpar[:])
