@@ -32,18 +32,26 @@ namespace gpflbm {
 // dendrite 0.670 ms against 0.689 / 0.715), although a CTA's march then
 // repeats a larger share of halo planes: the marches are short, the grid
 // is deep, and no general tile, whose lone march sets the step's tail,
-// runs long.
+// runs long.  FP64: 256 threads, since the paths need up to 255 (general) and
+// 128 (liquid) registers a thread; with 32 x 16 the compiler spills hundreds of
+// bytes a thread and an SM's one CTA waits on them (dendrite 100 x 90 x 96:
+// 2.34 ms a step with 32 x 16, 1.15 with 32 x 8; eutectic 91 x 79 x 66 half
+// solid: 2.94, 1.47; 150 x 130 x 171 mostly melt, where the wider tile redoes
+// fewer halo columns: 4.29, 4.11).
 template <class Real>
-struct Block3D {
-  static constexpr int BX = 32, BY = 16, ZS = sizeof(Real) == 4 ? 6 : 16;
+struct Block3D;
+template <>
+struct Block3D<float> {
+  static constexpr int BX = 32, BY = 16, ZS = 6;
+};
+template <>
+struct Block3D<double> {
+  static constexpr int BX = 32, BY = 8, ZS = 16;
 };
 
 template <int NP, int NC, class Real, class Store, int QQ = 19, bool SHRINK = false>
 struct Step3D {
-  // FP64 with shrinkage needs more than the 128 registers that 512 threads have
-  // (eutectic 91 x 79 x 66: 3.3 against 1.7 ms a step)
-  static constexpr int BX = Block3D<Real>::BX, BY = SHRINK && sizeof(Real) == 8 ? 8 : Block3D<Real>::BY;
-  static constexpr int ZS = Block3D<Real>::ZS;
+  static constexpr int BX = Block3D<Real>::BX, BY = Block3D<Real>::BY, ZS = Block3D<Real>::ZS;
   static constexpr int NT = BX * BY, Q = QQ;  // D3Q19 or D3Q27
   static constexpr int NS = PhiStore<NP>::NS;
   // values of a phase-field face: two phases need the difference of their two
