@@ -99,14 +99,9 @@ gpflbm_status cuda_fail(gpflbm_t h, cudaError_t e, const char* where) {
 }
 
 // The kernel table the time steps use: the extended model's when a pair of
-// the problem's phases has a nonzero tilt, an equilibrium composition depends
-// on temperature, or, in 3D with three or four phases, the gradient energy is
-// anisotropic without shrinkage (the plain kernels leave that out there, see
-// general_tile).
-const Ops* stepper(gpflbm_t h) {
-  const bool aniso = h->D == 3 && h->NP > 2 && !h->pf.shrink && !h->pd.shrink && (h->pf.aniso || h->pd.aniso);
-  return h->pf.tilted || h->pf.tdep || aniso ? h->ops_ext : h->ops;
-}
+// the problem's phases has a nonzero tilt or an equilibrium composition
+// depends on temperature.
+const Ops* stepper(gpflbm_t h) { return h->pf.tilted || h->pf.tdep ? h->ops_ext : h->ops; }
 
 // Record the caller's stream's progress for asynchronous loads, once per
 // run of read-only calls (see gpflbm_s::ev_mark).

@@ -140,6 +140,11 @@ struct Impl {
       if (e == cudaSuccess)
         e = cudaFuncSetAttribute(step3d_kernel<NP, NC, Real, Store, true, Q, EXT>,
                                  cudaFuncAttributeMaxDynamicSharedMemorySize, (int)SS::bytes);
+      if constexpr (NP > 2) {
+        if (e == cudaSuccess)
+          e = cudaFuncSetAttribute(step3d_kernel<NP, NC, Real, Store, false, Q, EXT, true>,
+                                   cudaFuncAttributeMaxDynamicSharedMemorySize, (int)step3d_bytes);
+      }
       if constexpr (!S3::ONE_LAUNCH) {
         if (e == cudaSuccess)
           e = cudaFuncSetAttribute(step3d_liquid_kernel<NP, NC, Real, Store, Q, EXT>,
@@ -186,6 +191,8 @@ struct Impl {
       if (P.shrink)  // (no liquid dispatch: every tile takes the general path)
         step3d_kernel<NP, NC, Real, Store, true, Q, EXT>
             <<<dim3((P.n[0] + SS::OX - 1) / SS::OX, (P.n[1] + SS::OY - 1) / SS::OY, gz), SS::NT, SS::bytes, s>>>(P, sio);
+      else if (NP > 2 && P.aniso)
+        step3d_kernel<NP, NC, Real, Store, false, Q, EXT, (NP > 2)><<<grid, S3::NT, step3d_bytes, s>>>(P, sio);
       else
         step3d_kernel<NP, NC, Real, Store, false, Q, EXT><<<grid, S3::NT, step3d_bytes, s>>>(P, sio);
       // the tiles whose reach is pure liquid (step3d_kernel returned there)

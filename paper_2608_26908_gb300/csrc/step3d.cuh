@@ -113,7 +113,12 @@ struct Step3DIO {
 // moves after its phase-field update (its populations are read again then).
 // The general path for one tile: xy tile (bx, by) of a gxt x gyt tiling,
 // z segment bz.  The kernels that run it are at the end of step3d_liquid.cuh.
-template <int NP, int NC, class Real, class Store, bool SHRINK, int QQ, bool EXT>
+// ANISO: three and four phases with an anisotropic gradient energy.  The code
+// of a plane is larger than the instruction cache, and the waits for
+// instructions are the general path's first stall: with the anisotropic
+// stencils beside the isotropic ones the isotropic eutectic 150 x 130 x 171 half
+// solid takes 481 us of general path a step, without them 436.
+template <int NP, int NC, class Real, class Store, bool SHRINK, int QQ, bool EXT, bool ANISO>
 __device__ __forceinline__ void general_tile(const DevParams<Real>& P, const Step3DIO& io, int bx, int by, int bz,
                                              int gxt, int gyt) {
   using S = Step3D<NP, NC, Real, Store, QQ, SHRINK>;
@@ -165,13 +170,8 @@ __device__ __forceinline__ void general_tile(const DevParams<Real>& P, const Ste
     else
       return P.ceq[a][i];
   };
-  // Three and four phases: the plain kernels are for isotropic problems, and an
-  // anisotropic one takes the extended model's (the launcher's choice).  The
-  // code of a plane is larger than the instruction cache, and the waits for
-  // instructions are the general path's first stall; with the anisotropic
-  // stencils in it the eutectic 150 x 130 x 171 half solid takes 481 us of
-  // general path a step, without them 436.
-  const bool aniso = (NP == 2 || EXT || SHRINK) && P.aniso != 0;
+  // (three and four phases: pf_face and the update beside it are isotropic)
+  const bool aniso = NP == 2 && P.aniso != 0;
   const bool has_walls = (P.wall[0] | P.wall[1] | P.wall[2]) != 0;  // obstacle rows
   // vertical index of a plane the kernel reads: folded on the whole grid
   // (walls mirror, periodic wraps), then kept inside the planes the buffers
@@ -268,6 +268,7 @@ __device__ __forceinline__ void general_tile(const DevParams<Real>& P, const Ste
   // copy of the code with d at run time ends the waits for instructions, but
   // executes a quarter more of them, 419 against 396 us on the grown eutectic.)
   constexpr int NF = S::NF;
+  constexpr bool DEFINITION = SHRINK || ANISO;  // the form of pf_flux
   auto pf_face = [&](int pa, int ia, int d, bool closed, Real* fl) {
 #pragma unroll
     for (int a = 0; a < NF; ++a) fl[a] = Real(0);
@@ -312,28 +313,20 @@ __device__ __forceinline__ void general_tile(const DevParams<Real>& P, const Ste
       const Real g2 = aniso ? Real(0.25) * (f[ap] + f[bp] - f[am] - f[bm]) : Real(0);
       fl[0] = flux(0, 1, f[B] - f[A], g1, g2);
     } else {
-      // A phase whose mask bit is clear in every cell the stencil reads is
-      // exactly 0 there, and every pair it belongs to contributes exactly 0.
-      Real pf[NP], gn[NP], g1[NP], g2[NP];
+      // (a phase that is 0 in both cells has q = 0 in every pair: exactly 0)
+      Real pf[NP], gn[NP];
 #pragma unroll
       for (int a = 0; a < NP; ++a) {
         const Real* f = s_phi + a * C2;
         const Real va = f[A], vb = f[B];
         pf[a] = Real(0.5) * (va + vb);
         gn[a] = vb - va;
-        g1[a] = g2[a] = Real(0);
-        if (aniso) {
-          g1[a] = Real(0.25) * (f[A + st] + f[B + st] - f[A - st] - f[B - st]);
-          g2[a] = Real(0.25) * (f[ap] + f[bp] - f[am] - f[bm]);
-        }
       }
 #pragma unroll
       for (int a = 0; a < NP; ++a)
 #pragma unroll
         for (int b = a + 1; b < NP; ++b) {
-          if ((NP == 2 || EXT) && (grp & ((1u << a) | (1u << b))) != ((1u << a) | (1u << b))) continue;
-          const Real gv = P.gamma[a][b] * flux(a, b, pf[a] * gn[b] - pf[b] * gn[a], pf[a] * g1[b] - pf[b] * g1[a],
-                                               pf[a] * g2[b] - pf[b] * g2[a]);
+          const Real gv = P.gamma[a][b] * (Real(2) * (pf[a] * gn[b] - pf[b] * gn[a]));
           fl[a] -= pf[b] * gv;
           fl[b] += pf[a] * gv;
         }
@@ -344,7 +337,10 @@ __device__ __forceinline__ void general_tile(const DevParams<Real>& P, const Ste
   // of either: another rounding of the update is a thousand times larger in the
   // force, and flips the stored rounding of 16-bit populations.  So this variant
   // evaluates the fluxes phase by phase, in the order of the definition (A and B
-  // are cells ia, ib of planes pa, pb).
+  // are cells ia, ib of planes pa, pb).  So does ANISO, where a pair with a phase
+  // absent from the stencil is too dear to evaluate (eutectic 150 x 130 x 171
+  // half solid in FP32, a step: pf_face with the anisotropic stencils 797 us,
+  // this form 519).
   auto pf_flux = [&](int pa, int ia, int pb, int ib, int d, bool closed, Real* fl) {
 #pragma unroll
     for (int a = 0; a < NP; ++a) fl[a] = Real(0);
@@ -498,6 +494,11 @@ __device__ __forceinline__ void general_tile(const DevParams<Real>& P, const Ste
 
     // C. phase field of plane C where phases mix
     const bool pfC = C >= z0 - 1 && C <= z0 + ZS;
+    // ANISO takes the first plane's lower z-face in the iteration before, by the
+    // code of the other z-faces: a face between two slabs is the last of the one
+    // and the first of the other, and the compiler rounds two copies of pf_flux
+    // differently.  (A slab's bits are the whole grid's; shrinkage has no slabs.)
+    const bool below = ANISO && !SHRINK && C == z0 - 2;
     Real out[NP];
     bool mixed = false, multi = false;
     unsigned act = 0;
@@ -513,9 +514,9 @@ __device__ __forceinline__ void general_tile(const DevParams<Real>& P, const Ste
     act = xy_m1 | xy_0 | xy_l;  // the 3x3x3 neighbourhood of plane C
     xy_m1 = xy_0;
     xy_0 = xy_l;
+    if (pfC || below) mixed = __popc(act) >= 2;
     if (pfC) {
       const int fzc = vz(C);
-      mixed = __popc(act) >= 2;
       multi = mixed && !(has_walls && obstacle(P, fx, fy, fzc));
 #pragma unroll
       for (int a = 0; a < NP; ++a) out[a] = PH(C, a, r2);
@@ -525,11 +526,11 @@ __device__ __forceinline__ void general_tile(const DevParams<Real>& P, const Ste
     // plane (and the z-face above it) is exactly zero.
     // (planes C-1, C and L all liquid: nothing mixes, and the CTA knows it
     // without another barrier)
-    if ((liq_hist & 7u) == 7u || !__syncthreads_or(pfC && mixed)) {
+    if ((liq_hist & 7u) == 7u || !__syncthreads_or(mixed)) {
 #pragma unroll
       for (int a = 0; a < NF; ++a) pfz_hi[a] = Real(0);
     } else {
-      if constexpr (SHRINK) {
+      if constexpr (DEFINITION) {
       if (pfC) {
         // in-plane faces of plane C into shared memory
         Real fl[NP];
@@ -537,11 +538,18 @@ __device__ __forceinline__ void general_tile(const DevParams<Real>& P, const Ste
         pf_flux(C, r2, C, r2 + 1, 0, cx_hi, fl);
 #pragma unroll
         for (int a = 0; a < NP; ++a) s_flux[a * (S::PFX + S::PFY) + ty * (BX + 1) + tx + 1] = fl[a];
-        if (tx == 0) {
-          const bool cx_lo = P.bc[0] == kWall && (gx == 0 || gx == nx);
-          pf_flux(C, r2 - 1, C, r2, 0, cx_lo, fl);
+        // The first face of every row by the lanes of one warp (a lane of each
+        // row's own warp costs every warp a face: anisotropic eutectic
+        // 64 x 60 x 66 in FP32, 164 us a step, 154 so), but not where registers
+        // are short (shrinkage, dendrite 150 x 130 x 171: 312 us, 319 so; turned
+        // axes, eutectic 150 x 130 x 171: 657 us, 708 so).
+        constexpr bool OWN = SHRINK || EXT;
+        if (OWN ? tx == 0 : tid >= NT - BY) {
+          const int j = OWN ? ty : tid - (NT - BY), first = OWN ? gx : x0 - 1;
+          const bool cx_lo = P.bc[0] == kWall && (first == 0 || first == nx);
+          pf_flux(C, (j + 1) * W2, C, (j + 1) * W2 + 1, 0, cx_lo, fl);
 #pragma unroll
-          for (int a = 0; a < NP; ++a) s_flux[a * (S::PFX + S::PFY) + ty * (BX + 1)] = fl[a];
+          for (int a = 0; a < NP; ++a) s_flux[a * (S::PFX + S::PFY) + j * (BX + 1)] = fl[a];
         }
         const bool cy_hi = P.bc[1] == kWall && (gy + 1 == 0 || gy + 1 == ny);
         pf_flux(C, r2, C, r2 + W2, 1, cy_hi, fl);
@@ -553,10 +561,12 @@ __device__ __forceinline__ void general_tile(const DevParams<Real>& P, const Ste
 #pragma unroll
           for (int a = 0; a < NP; ++a) s_flux[a * (S::PFX + S::PFY) + S::PFX + tx] = fl[a];
         }
-        // z-faces of this column: (C, C+1), and (C-1, C) on the first plane
+      }
+      // z-faces of this column: (C, C+1), and (C-1, C) on the first plane
+      if (pfC || below) {
         const bool cz_hi = P.bc[2] == kWall && (C + 1 == 0 || C + 1 == nz);
         pf_flux(C, r2, C + 1, r2, 2, cz_hi, pfz_hi);
-        if (C == z0 - 1) {
+        if (SHRINK && C == z0 - 1) {
           const bool cz_lo = P.bc[2] == kWall && (C == 0 || C == nz);
           pf_flux(C - 1, r2, C, r2, 2, cz_lo, pfz_lo);
         }
@@ -616,7 +626,7 @@ __device__ __forceinline__ void general_tile(const DevParams<Real>& P, const Ste
         Real mu[NC];
 #pragma unroll
         for (int i = 0; i < NC; ++i) mu[i] = s_mu[(slot2(C) * NC + i) * NT + tid];
-        if constexpr (SHRINK) {  // in the order of the definition, see pf_flux
+        if constexpr (DEFINITION) {  // see pf_flux
           Real div[NP], gc[NP][3];
 #pragma unroll
           for (int a = 0; a < NP; ++a) {
@@ -722,51 +732,29 @@ __device__ __forceinline__ void general_tile(const DevParams<Real>& P, const Ste
                         : (t == 1 ? Real(0.5) * (PH(C, a, r2 + W2) - PH(C, a, r2 - W2))
                                   : Real(0.5) * (PH(C + 1, a, r2) - PH(C - 1, a, r2)));
         };
-        // the gradient energy's centre terms
-        Real dadphi[NP];
+        // the gradient energy's centre terms: dA/dq = 2 q, q_ab = phi_a g_b -
+        // phi_b g_a, by the products g_a . g_b
+        Real G[NP][NP], dadphi[NP];
 #pragma unroll
         for (int a = 0; a < NP; ++a) dadphi[a] = Real(0);
-        if (!aniso) {
-          // dA/dq = 2 q, q_ab = phi_a g_b - phi_b g_a: by the products g_a . g_b
-          Real G[NP][NP];
 #pragma unroll
-          for (int t = 0; t < 3; ++t) {
-            Real g[NP];
+        for (int t = 0; t < 3; ++t) {
+          Real g[NP];
 #pragma unroll
-            for (int a = 0; a < NP; ++a) g[a] = grad(a, t);
-#pragma unroll
-            for (int a = 0; a < NP; ++a)
-#pragma unroll
-              for (int b = a; b < NP; ++b) G[a][b] = t == 0 ? g[a] * g[b] : G[a][b] + g[a] * g[b];
-          }
+          for (int a = 0; a < NP; ++a) g[a] = grad(a, t);
 #pragma unroll
           for (int a = 0; a < NP; ++a)
 #pragma unroll
-            for (int b = a + 1; b < NP; ++b) {
-              const Real g2 = Real(2) * P.gamma[a][b];
-              dadphi[a] += g2 * (ph[a] * G[b][b] - ph[b] * G[a][b]);
-              dadphi[b] += g2 * (ph[b] * G[a][a] - ph[a] * G[a][b]);
-            }
-        } else {
-          Real gc[NP][3];
-#pragma unroll
-          for (int a = 0; a < NP; ++a)
-#pragma unroll
-            for (int t = 0; t < 3; ++t) gc[a][t] = grad(a, t);
-#pragma unroll
-          for (int a = 0; a < NP; ++a)
-#pragma unroll
-            for (int b = a + 1; b < NP; ++b) {
-              const Real gab = P.gamma[a][b];
-              if (gab == Real(0) || (act & ((1u << a) | (1u << b))) != ((1u << a) | (1u << b))) continue;
-              Real q[3], v[3];
-#pragma unroll
-              for (int t = 0; t < 3; ++t) q[t] = ph[a] * gc[b][t] - ph[b] * gc[a][t];
-              dAdq_vec_pair<3, EXT>(P, a, b, q, v);
-              dadphi[a] += gab * (v[0] * gc[b][0] + v[1] * gc[b][1] + v[2] * gc[b][2]);
-              dadphi[b] -= gab * (v[0] * gc[a][0] + v[1] * gc[a][1] + v[2] * gc[a][2]);
-            }
+            for (int b = a; b < NP; ++b) G[a][b] = t == 0 ? g[a] * g[b] : G[a][b] + g[a] * g[b];
         }
+#pragma unroll
+        for (int a = 0; a < NP; ++a)
+#pragma unroll
+          for (int b = a + 1; b < NP; ++b) {
+            const Real g2 = Real(2) * P.gamma[a][b];
+            dadphi[a] += g2 * (ph[a] * G[b][b] - ph[b] * G[a][b]);
+            dadphi[b] += g2 * (ph[b] * G[a][a] - ph[a] * G[a][b]);
+          }
         Real psi[NP];
 #pragma unroll
         for (int b = 0; b < NP; ++b) {
@@ -878,6 +866,8 @@ __device__ __forceinline__ void general_tile(const DevParams<Real>& P, const Ste
       }
       s_chg[slot2(C) * NT + tid] = changed ? 1 : 0;
       s_hl[slot2(C) * NT + tid] = interp_h<NP>(out, 0);
+    }
+    if (pfC || below) {
 #pragma unroll
       for (int a = 0; a < NF; ++a) pfz_lo[a] = pfz_hi[a];
     }

@@ -298,7 +298,7 @@ __device__ __forceinline__ void liquid_tiles(const DevParams<Real>& P, const Ste
 // would hold the liquid tiles to its occupancy; three or four phases: its
 // shared memory, see ONE_LAUNCH) step3d_kernel takes the general tiles and
 // step3d_liquid_kernel, launched after it, the others.
-template <int NP, int NC, class Real, class Store, bool SHRINK = false, int QQ = 19, bool EXT = false>
+template <int NP, int NC, class Real, class Store, bool SHRINK = false, int QQ = 19, bool EXT = false, bool ANISO = false>
 __global__ void __launch_bounds__(Step3D<NP, NC, Real, Store, QQ, SHRINK>::NT, Step3D<NP, NC, Real, Store, QQ>::MIN_CTAS)
     step3d_kernel(const DevParams<Real> P, const Step3DIO io) {
   using S = Step3D<NP, NC, Real, Store, QQ, SHRINK>;
@@ -314,7 +314,7 @@ __global__ void __launch_bounds__(Step3D<NP, NC, Real, Store, QQ, SHRINK>::NT, S
   }
   const int bz = blockIdx.z;
   if (P.liq_dispatch && liquid_reach<ZS>(P, io.flags_in, bx, by, P.v_lo + bz * ZS, gxt, gyt)) return;
-  general_tile<NP, NC, Real, Store, SHRINK, QQ, EXT>(P, io, bx, by, bz, gxt, gyt);
+  general_tile<NP, NC, Real, Store, SHRINK, QQ, EXT, ANISO>(P, io, bx, by, bz, gxt, gyt);
 }
 
 template <int NP, int NC, class Real, class Store, int QQ = 19, bool EXT = false>

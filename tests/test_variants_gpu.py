@@ -1,11 +1,13 @@
 """Every variant of the step kernels that a size or a model switches to,
-against the FP64 oracle: the 3D tiles in FP64 at their edges, with each model.
+against the FP64 oracle: the 3D tiles in FP64 at their edges, with each model,
+and the anisotropic 3D kernels of three and four phases.
 Tolerances of the plain step after 100 steps (test_parity_gpu): FP64 1e-10 (U
 and the population deviations 1e-8), FP32 1e-5."""
+import numpy as np
 import pytest
 
 from parity import errors
-from paper_2608_26908_gb300 import inputs
+from paper_2608_26908_gb300 import gpflbm, inputs, slabs
 
 pytestmark = pytest.mark.gpu
 
@@ -52,3 +54,67 @@ def test_3d_fp64(name, size, lattice, model):
     if name == "eutectic3d":
         sc["init"]["height"] = 9
     _check(_model(sc, model), 25)
+
+
+def _eutectic3d(size, prec, phases, solutes, lattice=19):
+    sc = inputs.scenario("eutectic3d", **dict(zip(("nx", "ny", "nz"), size)), precision=prec)
+    sc["grid"]["lattice"] = lattice
+    sc["init"]["height"] = 12
+    sc["n_phases"], sc["n_solutes"] = phases, solutes
+    return sc
+
+
+@pytest.mark.parametrize("prec,phases,solutes,lattice,model", [
+    ("fp32", 4, 2, 19, "aniso"),
+    ("fp32", 3, 1, 19, "aniso"),
+    ("fp64", 4, 1, 19, "aniso"),
+    ("fp64", 3, 2, 27, "aniso"),
+    ("fp32", 4, 2, 27, "aniso"),
+    ("fp32", 4, 2, 19, "tilt"),
+    ("fp64", 3, 1, 19, "tilt"),
+    ("fp64", 4, 2, 19, "combined"),
+])
+def test_3d_anisotropic(prec, phases, solutes, lattice, model):
+    _check(_model(_eutectic3d((33, 29, 31), prec, phases, solutes, lattice), model), 25)
+
+
+@pytest.mark.parametrize("prec,phases,solutes,lattice,model", [
+    ("fp32_bf16", 4, 2, 19, "aniso"),
+    ("fp32", 3, 1, 19, "aniso"),
+    ("fp64", 4, 1, 19, "aniso"),
+    ("fp32", 3, 2, 27, "aniso"),
+    ("fp32", 4, 2, 19, "tilt"),
+    ("fp64", 3, 1, 27, "tilt"),
+    ("fp32_f16", 4, 2, 19, "ceqT"),
+    ("fp64", 4, 2, 19, "plain"),
+    ("fp32", 3, 1, 19, "plain"),
+    ("fp32_bf16", 2, 2, 19, "aniso"),
+    ("fp64", 2, 1, 27, "tilt"),
+])
+def test_3d_slabs_match_the_whole_grid(prec, phases, solutes, lattice, model):
+    """The same bits, also after a change of parameters from isotropic ones
+    (another kernel of the same handle)."""
+    def scenario(m):
+        return _model(_eutectic3d((40, 34, 32), prec, phases, solutes, lattice), m)
+
+    sc = scenario(model)
+    phi0, mu0 = inputs.initial_state(sc)
+    layer, steps = 40 * 34, 6
+    whole = gpflbm.Sim(scenario("plain"))
+    whole.set_state(phi0, mu0)
+    whole.step(4)
+    whole.set_params(sc)
+    whole.set_state(phi0, mu0)
+    whole.step(steps)
+    ref = whole.fields(("phi", "mu", "f"))
+    runs = []
+    for r, (v0, n) in enumerate([(0, 9), (9, 2), (11, 21)]):
+        sim = gpflbm.Sim(sc, slab=(v0, n))
+        sim.set_state(*[a.reshape(-1, 32 * layer)[:, v0 * layer:(v0 + n) * layer].reshape(-1) for a in (phi0, mu0)])
+        runs.append((v0, n, slabs.Slab(sim, r, 3)))
+    for _ in range(steps):
+        slabs.step_all([s for _, _, s in runs])
+    for v0, n, s in runs:
+        got = s.sim.fields(("phi", "mu", "f"))
+        for k in got:
+            np.testing.assert_array_equal(got[k], ref[k][:, v0 * layer:(v0 + n) * layer], err_msg=k)
