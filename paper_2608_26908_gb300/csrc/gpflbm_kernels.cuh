@@ -873,11 +873,14 @@ __device__ __forceinline__ Real composition(const DevParams<Real>& P, const Real
 // Each thread takes V consecutive cells of a row (nx a multiple of V and, for
 // V > 1, every destination 16-byte aligned), reads all it needs of them before
 // its first store, and runs a grid-stride loop over a grid the launcher caps
-// (see load_state_kernel).  Bound by HBM: phi, mu, f and u of 256^3 cells
-// (3.2 GB read and written) take 466 us, 6.8 TB/s; one cell a thread with
-// each store after its load on two CTAs an SM, which this replaces, 949 us.
+// (see load_state_kernel).  FP32 is bound by HBM: phi, mu, f and u of 256^3
+// cells (two phases, one solute: 3.09 GB read and written) take 466 us, 6.6 TB/s;
+// one cell a thread with each store after its load on two CTAs an SM, which
+// this replaces, 949 us.  FP64 is bound by its issue, and takes 128 registers a
+// thread: with 64 they spill (eutectic 97 x 90 x 88, every field: 283 us against
+// 266).
 template <int D, int Q, int NP, int NC, class Real, class Store, class Out, int V>
-__global__ void __launch_bounds__(256, V == 1 ? 4 : 2)
+__global__ void __launch_bounds__(256, V == 1 && sizeof(Real) == 4 ? 4 : 2)
     fields_kernel(const DevParams<Real> P, const Real* __restrict__ phi, const Real* __restrict__ mu_in,
                   const Store* __restrict__ f, const double* __restrict__ clock, Out* __restrict__ o_phi,
                   Out* __restrict__ o_mu, Out* __restrict__ o_c, Out* __restrict__ o_f, Out* __restrict__ o_rho,

@@ -254,7 +254,9 @@ struct Impl {
   static cudaError_t fields(const void* params, const FieldsIO& io, cudaStream_t s) {
     const DevParams<Real>& P = *static_cast<const DevParams<Real>*>(params);
     const long long cells = (long long)P.n[0] * P.n[1] * P.n[2];
-    constexpr int V = 16 / (int)sizeof(Real);  // one 16-byte word of each plane
+    // one 16-byte word of each plane; D3Q27 in FP64 one cell (two cells' values do
+    // not fit 128 registers: 100 x 90 x 96, every field, 316 us against 308)
+    constexpr int V = sizeof(Real) == 8 && Q == 27 ? 1 : 16 / (int)sizeof(Real);
     auto al16 = [](const void* p) { return (reinterpret_cast<uintptr_t>(p) & 15u) == 0; };
     const int threads = 256;
     // A grid too small to give every SM a CTA of V cells a thread is bound by a
