@@ -65,6 +65,7 @@ struct gpflbm_s {
   // for the load.  Every entry point other than the read-only ones bumps mut.
   cudaStream_t xfer;
   cudaEvent_t ev_mark, ev_loaded;
+  bool link_load;  // the state came by an asynchronous load from host memory, not written back since
   unsigned long long mut, marked;
   // device parameters in the arithmetic type (only one is used)
   DevParams<double> pd;
@@ -819,6 +820,7 @@ gpflbm_status gpflbm_set_state(gpflbm_t h, const void* phi, const void* mu, cons
     if (e != cudaSuccess) return cuda_fail(h, e, "set_state: load");
     h->cur = to;
     h->t = t0;
+    h->link_load = !on_device;
     h->halo_fresh[0] = h->halo_fresh[1] = false;
     ++h->mut;
     return GPFLBM_OK;
@@ -843,6 +845,7 @@ gpflbm_status gpflbm_set_state(gpflbm_t h, const void* phi, const void* mu, cons
   }
   h->t = t0;
   h->has_state = true;
+  h->link_load = false;
   h->halo_fresh[0] = h->halo_fresh[1] = false;
   ++h->mut;
   return GPFLBM_OK;
@@ -1010,7 +1013,11 @@ gpflbm_status gpflbm_get_fields(gpflbm_t h, unsigned field_mask, void* const* ds
   }
   cudaError_t e;
   if (any_direct) {
+    // A loop that loads each state over the host link and writes its result to
+    // the device loads the next one beside this write-back.
     direct.link = !on_device;
+    direct.beside = h->link_load;
+    h->link_load = false;
     e = h->ops->fields(xparams(h), direct, s);
     if (e != cudaSuccess) return cuda_fail(h, e, "get_fields: kernel");
   }

@@ -37,7 +37,8 @@ struct FieldsIO {
   void* o_rho;
   void* o_u;
   void* o_dev;
-  bool link;  // a destination is host memory, written over the host link
+  bool link;    // a destination is host memory, written over the host link
+  bool beside;  // a load over the host link may run at the same time
 };
 
 struct Ops {
@@ -69,10 +70,13 @@ struct Ops {
 // Grid of the exchange kernels (state load, field write-back): a grid-stride
 // loop over `per_sm` CTAs of 256 threads per SM.  Two keep enough accesses in
 // flight for the host link and leave room on every SM for the other
-// of the two kernels, which may run at the same time on another stream; between
-// device buffers nothing runs beside them, and HBM wants more loads in
-// flight (1001^2 cells, one a thread: the load 21.5 us with two, 14.0 us with
-// eight).
+// of the two kernels, which may run at the same time on another stream (a
+// write-back to the device whose CTAs fill the chip holds a load over the link
+// back until it ends: 256^3, step, write-back and load 7.77 ms, 7.38 with two;
+// one that leaves room does not: 500 x 301 in FP64, 138 us, 146).  Between
+// device buffers HBM wants more loads in flight, beside each other too (1001^2
+// cells, one a thread: the load 21.5 us with two, 14.0 us with eight; 256^3,
+// step, write-back and load beside it: 1.90 ms, 1.59).
 constexpr int kLinkCtas = 2, kDeviceCtas = 8;
 inline unsigned exchange_blocks(long long items, int threads, int per_sm) {
   static int sms = 0;
@@ -265,9 +269,10 @@ struct Impl {
     // Over the host link the words gain nothing, and their registers leave the
     // load beside the write-back too little of an SM (two CTAs an SM: eutectic3d
     // end to end 1.82k -> 1.56k MLUPS; one: eutectic2d 3.31k -> 3.24k).
-    const bool vec = !io.link && P.n[0] % V == 0 && cells / V >= 152 * threads && al16(io.o_phi) && al16(io.o_mu) && al16(io.o_c) &&
+    const bool link = io.link || (io.beside && cells >= 152LL * kDeviceCtas * threads);
+    const bool vec = !link && P.n[0] % V == 0 && cells / V >= 152 * threads && al16(io.o_phi) && al16(io.o_mu) && al16(io.o_c) &&
                      al16(io.o_f) && al16(io.o_rho) && al16(io.o_u) && al16(io.o_dev);
-    const unsigned blocks = exchange_blocks(vec ? cells / V : cells, threads, io.link ? kLinkCtas : kDeviceCtas);
+    const unsigned blocks = exchange_blocks(vec ? cells / V : cells, threads, link ? kLinkCtas : kDeviceCtas);
     auto go = [&](auto kernel) {
       kernel<<<blocks, threads, 0, s>>>(
           P, static_cast<const Real*>(io.phi), static_cast<const Real*>(io.mu), static_cast<const Store*>(io.f),

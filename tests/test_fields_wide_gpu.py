@@ -56,3 +56,23 @@ def test_words_and_single_cells_read_the_same_fields(name, size, prec, lattice):
     wide, single = _read(sim, 0), _read(sim, 1)
     for n, a, b in zip(NAMES, wide, single):
         np.testing.assert_array_equal(a, b, err_msg=n)
+
+
+@pytest.mark.parametrize("size", [dict(nx=80, ny=64, nz=64), dict(nx=73, ny=66, nz=65), dict(nx=40, ny=36, nz=20)])
+def test_write_back_after_an_asynchronous_host_load(size):
+    """The write-back that expects another load over the host link beside it
+    (the first after an asynchronous load from host memory, on a grid that
+    fills the chip) gives the bits of the next one, which does not."""
+    import torch
+
+    sc = inputs.scenario("dendrite3d", precision="fp32", **size)
+    sim = gpflbm.Sim(sc)
+    state = [torch.as_tensor(a, dtype=torch.float32).pin_memory() for a in inputs.initial_state(sc)]
+    sim.set_state(*state)
+    st = gpflbm.lib().gpflbm_set_state(sim.h, state[0].data_ptr(), state[1].data_ptr(), None, gpflbm.ASYNC, 0,
+                                       ctypes.c_void_p(torch.cuda.current_stream().cuda_stream))
+    assert st == gpflbm.OK
+    sim.step(4)
+    first, second = _read(sim, 0), _read(sim, 0)
+    for n, a, b in zip(NAMES, first, second):
+        np.testing.assert_array_equal(a, b, err_msg=n)
