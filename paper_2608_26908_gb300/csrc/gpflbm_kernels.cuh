@@ -440,26 +440,32 @@ __device__ __forceinline__ Real interp_dh(const Real* p, int b, int a) {
   return Real(2) * p[b] * s;
 }
 
-// drv_a = sum_b psi_b dh_b/dphi_a: with w_b = psi_b phi_b and T = sum phi,
-//   psi_a (6 phi_a (1 - phi_a) + 2 E_a) + 2 sum_{b != a} w_b (T - phi_a - phi_b),
-// E_a = sum_{b<g; b,g != a} phi_b phi_g (a fifth of the operations of
-// interp_dh pair by pair).
+// drv_a = sum_b psi_b dh_b/dphi_a: with w_b = psi_b phi_b,
+//   psi_a (6 phi_a (1 - phi_a) + 2 E_a) + 2 sum_{b != a} w_b sum_{g != a,b} phi_g,
+// E_a = sum_{b<g; b,g != a} phi_b phi_g (a third of the operations of
+// interp_dh pair by pair).  The sums run over the other phases: as differences
+// of sums over all of them they would leave a trace phase beside a nearly pure
+// one the rounding of terms of order psi, where its own are of order
+// phi_a psi.
 template <int NP, class Real>
-__device__ __forceinline__ void driving_force(const Real* p, const Real* psi, Real* drv) {
-  Real w[NP], T = Real(0), W = Real(0), X = Real(0), e2 = Real(0);
+__host__ __device__ __forceinline__ void driving_force(const Real* p, const Real* psi, Real* drv) {
+  Real w[NP];
 #pragma unroll
-  for (int b = 0; b < NP; ++b) {
-    w[b] = psi[b] * p[b];
-    e2 += T * p[b];
-    T += p[b];
-    W += w[b];
-    X += w[b] * p[b];
-  }
+  for (int b = 0; b < NP; ++b) w[b] = psi[b] * p[b];
 #pragma unroll
   for (int a = 0; a < NP; ++a) {
-    const Real t = T - p[a];  // the other phases
-    const Real cross = t * (W - w[a]) - (X - w[a] * p[a]);
-    const Real E = e2 - p[a] * t;
+    Real E = Real(0), cross = Real(0), before = Real(0);  // before: the phases below b
+#pragma unroll
+    for (int b = 0; b < NP; ++b) {
+      if (b == a) continue;
+      Real t = before;
+#pragma unroll
+      for (int g = b + 1; g < NP; ++g)
+        if (g != a) t += p[g];
+      cross += w[b] * t;
+      E += before * p[b];
+      before += p[b];
+    }
     drv[a] = psi[a] * (Real(6) * p[a] * (Real(1) - p[a]) + Real(2) * E) + Real(2) * cross;
   }
 }
