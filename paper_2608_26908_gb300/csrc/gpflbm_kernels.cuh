@@ -1186,35 +1186,37 @@ __global__ void __launch_bounds__(kRedThreads, sizeof(Real) == 4 ? 4 : 2)
         if (a == b) inv = P.inv2A[b];
       return __dadd_rn(ce, __dmul_rn(m64[i], inv));
     };
+    // The phases present, in ascending order, in slots (the others at 0):
+    // a phase at 0 has h = 0 and adds 0 to every sum, exactly.
+    using Slot = typename std::conditional<NP == 2, double, Real>::type;  // (phi_0 of two phases: FP64)
+    Slot q[NP];
+    int id[NP], n = 0;
+#pragma unroll
+    for (int j = 0; j < NP; ++j) {
+      q[j] = Slot(0);
+      id[j] = 0;
+    }
+#pragma unroll
+    for (int a = 0; a < NP; ++a) {
+      Slot pa;
+      if (NP == 2)
+        pa = a == 0 ? (ps[0] == Real(0) ? Slot(1) : Slot(__dsub_rn(1.0, widen(ps[0])))) : Slot(widen(ps[0]));
+      else
+        pa = Slot(ps[NP == 2 ? 0 : a]);
+      if (pa == Slot(0)) continue;
+#pragma unroll
+      for (int j = 0; j <= a; ++j)
+        if (n == j) {
+          q[j] = pa;
+          id[j] = a;
+        }
+      ++n;
+    }
+    // (the lanes with a cell left vote, before the branches below part them)
+    const unsigned left = cells - (x - (threadIdx.x & 31u));
+    const bool pure = __all_sync(left >= 32u ? ~0u : (1u << left) - 1u, fm && n == 1 && q[0] == Slot(1));
     if (fm) {
-      // The phases present, in ascending order, in slots (the others at 0):
-      // a phase at 0 has h = 0 and adds 0 to every sum, exactly.
-      using Slot = typename std::conditional<NP == 2, double, Real>::type;  // (phi_0 of two phases: FP64)
-      Slot q[NP];
-      int id[NP], n = 0;
-#pragma unroll
-      for (int j = 0; j < NP; ++j) {
-        q[j] = Slot(0);
-        id[j] = 0;
-      }
-#pragma unroll
-      for (int a = 0; a < NP; ++a) {
-        Slot pa;
-        if (NP == 2)
-          pa = a == 0 ? (ps[0] == Real(0) ? Slot(1) : Slot(__dsub_rn(1.0, widen(ps[0])))) : Slot(widen(ps[0]));
-        else
-          pa = Slot(ps[NP == 2 ? 0 : a]);
-        if (pa == Slot(0)) continue;
-#pragma unroll
-        for (int j = 0; j <= a; ++j)
-          if (n == j) {
-            q[j] = pa;
-            id[j] = a;
-          }
-        ++n;
-      }
-      const bool pure = n == 1 && q[0] == Slot(1);
-      if (__all_sync(__activemask(), pure)) {  // h is the unit vector, exactly
+      if (pure) {  // h is the unit vector, exactly
 #pragma unroll
         for (int i = 0; i < NC; ++i) acc[1 + i] = __dadd_rn(acc[1 + i], c_of(id[0], i));
         if (id[0] > 0) acc[NC + 1] = __dadd_rn(acc[NC + 1], 1.0);
