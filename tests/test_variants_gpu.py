@@ -1,12 +1,13 @@
 """Every variant of the step kernels that a size or a model switches to,
 against the FP64 oracle: the 3D tiles in FP64 at their edges, with each model,
-and the anisotropic 3D kernels of three and four phases.
+the anisotropic 3D kernels of three and four phases, both 2D tiles in FP64, and
+the two-segment march at a ragged end.
 Tolerances of the plain step after 100 steps (test_parity_gpu): FP64 1e-10 (U
 and the population deviations 1e-8), FP32 1e-5."""
 import numpy as np
 import pytest
 
-from parity import errors
+from parity import device_run, reference, rel_err
 from paper_2608_26908_gb300 import gpflbm, inputs, slabs
 
 pytestmark = pytest.mark.gpu
@@ -31,11 +32,13 @@ def _model(sc, model):
     return sc
 
 
-def _check(sc, steps, **kw):
-    errs = errors(sc, steps, **kw)[0]
-    for k, e in errs.items():
+def _check(sc, steps, **state):
+    ref = reference(sc, steps, **state)
+    sim, got = device_run(sc, steps, **state)
+    sim.close()
+    for k in ("phi", "mu", "c", "rho", "u", "dev"):
         tol = 1e-5 if sc["precision"] == "fp32" else (1e-8 if k in ("u", "dev") else 1e-10)
-        assert e <= tol, (k, e)
+        assert rel_err(got[k], ref[k]) <= tol, (k, rel_err(got[k], ref[k]))
 
 
 # FP64 tiles own 30 x 6 columns and march 16 planes
@@ -112,6 +115,70 @@ def test_3d_slabs_match_the_whole_grid(prec, phases, solutes, lattice, model):
         sim = gpflbm.Sim(sc, slab=(v0, n))
         sim.set_state(*[a.reshape(-1, 32 * layer)[:, v0 * layer:(v0 + n) * layer].reshape(-1) for a in (phi0, mu0)])
         runs.append((v0, n, slabs.Slab(sim, r, 3)))
+    for _ in range(steps):
+        slabs.step_all([s for _, _, s in runs])
+    for v0, n, s in runs:
+        got = s.sim.fields(("phi", "mu", "f"))
+        for k in got:
+            np.testing.assert_array_equal(got[k], ref[k][:, v0 * layer:(v0 + n) * layer], err_msg=k)
+
+
+def _case2d(nx, ny, phases, solutes):
+    """Stripes of every solid phase below a melt, with blurred edges."""
+    sc = inputs.scenario("eutectic2d", nx=nx, ny=ny, precision="fp64")
+    ternary = inputs.scenario("eutectic3d", nx=nx, ny=ny, nz=3)["params"]
+    for k in ("gamma", "ceq", "S", "A"):
+        sc["params"][k] = ternary[k]
+    sc["n_phases"], sc["n_solutes"] = phases, solutes
+    x, y = np.meshgrid(np.arange(nx), np.arange(ny))
+    phi = np.zeros((phases, ny, nx))
+    for a in range(1, phases):
+        phi[a] = (y < 40 + 5 * a) & (1 + (x // 11) % (phases - 1) == a)
+    phi[0] = 1.0 - phi[1:].sum(axis=0)
+    for _ in range(2):  # three-cell means: interfaces a few cells wide
+        phi = (np.roll(phi, 1, 2) + phi + np.roll(phi, -1, 2)) / 3.0
+        up, down = np.concatenate([phi[:, :1], phi[:, :-1]], 1), np.concatenate([phi[:, 1:], phi[:, -1:]], 1)
+        phi = (up + phi + down) / 3.0
+    mu = 0.02 * np.sin(np.arange(solutes * nx * ny) * 0.37)
+    return sc, phi.reshape(-1), mu
+
+
+# 32 x 8 tiles own 30 x 6 cells: 305 of them on 150 x 366 (the first grid of
+# large tiles), 304 on 480 x 114 (the last of small ones)
+@pytest.mark.parametrize("nx,ny", [(150, 366), (480, 114)])
+@pytest.mark.parametrize("phases,solutes,model", [
+    (2, 1, "plain"), (2, 2, "plain"), (3, 2, "plain"), (4, 1, "plain"),
+    (2, 2, "shrinkage"), (3, 1, "shrinkage"), (4, 2, "shrinkage"),
+    (2, 1, "tilt"), (4, 1, "tilt"),
+    (2, 2, "ceqT"), (3, 1, "ceqT"), (4, 2, "ceqT"),
+    (2, 1, "combined"), (3, 2, "combined"), (4, 2, "combined"),
+])
+def test_2d_fp64_on_both_sides_of_the_tile_rule(nx, ny, phases, solutes, model):
+    sc, phi0, mu0 = _case2d(nx, ny, phases, solutes)
+    _check(_model(sc, model), 12, phi0=phi0, mu0=mu0)
+
+
+@pytest.mark.parametrize("nz,phases", [(256, 2), (259, 2), (261, 4)])
+def test_two_segments_a_march_at_a_ragged_end(nz, phases):
+    """16-bit populations: 43 and 44 segments of six planes, marched by twos,
+    the last one ragged; the slabs, whose every tile is general, give the same
+    bits."""
+    sc = inputs.scenario("eutectic3d" if phases == 4 else "dendrite3d", nx=190, ny=180, nz=nz, precision="fp32_f16")
+    sc["params"]["gbeta_c"] = [2e-3, 1e-3]
+    # tiles of 30 x 14 columns; below 2000 CTAs a march takes one segment
+    assert (190 + 29) // 30 * ((180 + 13) // 14) * (((nz + 5) // 6 + 1) // 2) >= 2000
+    phi0, mu0 = inputs.initial_state(sc)
+    layer, steps = 190 * 180, 3
+    whole = gpflbm.Sim(sc)
+    whole.set_state(phi0, mu0)
+    whole.step(steps)
+    ref = whole.fields(("phi", "mu", "f"))
+    whole.close()
+    runs = []
+    for r, (v0, n) in enumerate([(0, 129), (129, nz - 129)]):
+        sim = gpflbm.Sim(sc, slab=(v0, n))
+        sim.set_state(*[a.reshape(-1, nz * layer)[:, v0 * layer:(v0 + n) * layer].reshape(-1) for a in (phi0, mu0)])
+        runs.append((v0, n, slabs.Slab(sim, r, 2)))
     for _ in range(steps):
         slabs.step_all([s for _, _, s in runs])
     for v0, n, s in runs:
