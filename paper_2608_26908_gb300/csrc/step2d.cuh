@@ -38,7 +38,7 @@ template <>
 struct Block2D<double, false> {
   static constexpr int BX = 32, BY = 8, MIN_CTAS = 4;
 };
-// FP64 grids too small to fill the chip (SMALL2D_BLOCKS below): an SM issues
+// FP64 grids too small to fill the chip (kSmall2DBlocks, gpflbm_ops.cuh): an SM issues
 // one FP64 warp instruction every 16 cycles, so the SM with the most warps on
 // the interface sets the step's time, and small tiles spread them.
 template <>
@@ -482,76 +482,76 @@ __global__ void __launch_bounds__(Step2D<NP, NC, Real, Store, SMALL>::NT, Step2D
         out[1] = u;
         out[0] = Real(1) - u;
       } else {
-      Real div[NP], gc[NP][2];
+        Real div[NP], gc[NP][2];
 #pragma unroll
-      for (int a = 0; a < NP; ++a) {
-        const Real* fa = s_flux + a * (S::PFX + S::PFY);
-        div[a] = (fa[ty * (BX + 1) + tx + 1] - fa[ty * (BX + 1) + tx]) +
-                 (fa[S::PFX + (ty + 1) * BX + tx] - fa[S::PFX + ty * BX + tx]);
-        gc[a][0] = Real(0.5) * (PH(a, r2 + 1) - PH(a, r2 - 1));
-        gc[a][1] = Real(0.5) * (PH(a, r2 + W2) - PH(a, r2 - W2));
-      }
-      Real dadphi[NP];
-#pragma unroll
-      for (int a = 0; a < NP; ++a) dadphi[a] = Real(0);
-#pragma unroll
-      for (int a = 0; a < NP; ++a)
-#pragma unroll
-        for (int b = a + 1; b < NP; ++b) {
-          // a phase absent from the 3x3 neighbourhood: q = 0, exactly 0
-          const Real gab = P.gamma[a][b];
-          if (gab == Real(0) || (act & ((1u << a) | (1u << b))) != ((1u << a) | (1u << b))) continue;
-          Real q[2], v[2];
-          q[0] = ph[a] * gc[b][0] - ph[b] * gc[a][0];
-          q[1] = ph[a] * gc[b][1] - ph[b] * gc[a][1];
-          dAdq_vec_pair<2, EXT>(P, a, b, q, v);
-          dadphi[a] += gab * (v[0] * gc[b][0] + v[1] * gc[b][1]);
-          dadphi[b] -= gab * (v[0] * gc[a][0] + v[1] * gc[a][1]);
+        for (int a = 0; a < NP; ++a) {
+          const Real* fa = s_flux + a * (S::PFX + S::PFY);
+          div[a] = (fa[ty * (BX + 1) + tx + 1] - fa[ty * (BX + 1) + tx]) +
+                   (fa[S::PFX + (ty + 1) * BX + tx] - fa[S::PFX + ty * BX + tx]);
+          gc[a][0] = Real(0.5) * (PH(a, r2 + 1) - PH(a, r2 - 1));
+          gc[a][1] = Real(0.5) * (PH(a, r2 + W2) - PH(a, r2 - W2));
         }
-      Real psi[NP];
+        Real dadphi[NP];
 #pragma unroll
-      for (int b = 0; b < NP; ++b) {
-        Real sv = P.S[b] * theta;
+        for (int a = 0; a < NP; ++a) dadphi[a] = Real(0);
 #pragma unroll
-        for (int i = 0; i < NC; ++i) sv -= mu[i] * mu[i] * P.inv4A[b] + mu[i] * ceq_of(b, i);
-        psi[b] = sv;
-      }
-      Real rate[NP];
+        for (int a = 0; a < NP; ++a)
 #pragma unroll
-      for (int a = 0; a < NP; ++a) {
-        Real obst = Real(0), drv = Real(0);
+          for (int b = a + 1; b < NP; ++b) {
+            // a phase absent from the 3x3 neighbourhood: q = 0, exactly 0
+            const Real gab = P.gamma[a][b];
+            if (gab == Real(0) || (act & ((1u << a) | (1u << b))) != ((1u << a) | (1u << b))) continue;
+            Real q[2], v[2];
+            q[0] = ph[a] * gc[b][0] - ph[b] * gc[a][0];
+            q[1] = ph[a] * gc[b][1] - ph[b] * gc[a][1];
+            dAdq_vec_pair<2, EXT>(P, a, b, q, v);
+            dadphi[a] += gab * (v[0] * gc[b][0] + v[1] * gc[b][1]);
+            dadphi[b] -= gab * (v[0] * gc[a][0] + v[1] * gc[a][1]);
+          }
+        Real psi[NP];
 #pragma unroll
         for (int b = 0; b < NP; ++b) {
-          if (b != a) obst += P.gamma[a][b] * ph[b];
-          drv += psi[b] * interp_dh<NP>(ph, b, a);
+          Real sv = P.S[b] * theta;
+#pragma unroll
+          for (int i = 0; i < NC; ++i) sv -= mu[i] * mu[i] * P.inv4A[b] + mu[i] * ceq_of(b, i);
+          psi[b] = sv;
         }
-        rate[a] = P.eps * (div[a] - dadphi[a]) - P.obst * obst - drv;
-      }
-      int na = 0;
-      Real lam = Real(0);
+        Real rate[NP];
 #pragma unroll
-      for (int a = 0; a < NP; ++a)
-        if (act & (1u << a)) {
-          lam += rate[a];
-          ++na;
+        for (int a = 0; a < NP; ++a) {
+          Real obst = Real(0), drv = Real(0);
+#pragma unroll
+          for (int b = 0; b < NP; ++b) {
+            if (b != a) obst += P.gamma[a][b] * ph[b];
+            drv += psi[b] * interp_dh<NP>(ph, b, a);
+          }
+          rate[a] = P.eps * (div[a] - dadphi[a]) - P.obst * obst - drv;
         }
-      lam = lam / Real(na);
-      Real uv[NP];
-      int m = 0;
+        int na = 0;
+        Real lam = Real(0);
 #pragma unroll
-      for (int a = 0; a < NP; ++a)
-        if (act & (1u << a)) uv[m++] = ph[a] + P.mob_eps * (rate[a] - lam);
-      if (NP == 2) {
-        Real sv = uv[1];
-        sv = sv < Real(0) ? Real(0) : (sv > Real(1) ? Real(1) : sv);
-        out[1] = sv;
-        out[0] = Real(1) - sv;
-      } else {
-        project_simplex<Real, NP>(uv, m);
-        m = 0;
+        for (int a = 0; a < NP; ++a)
+          if (act & (1u << a)) {
+            lam += rate[a];
+            ++na;
+          }
+        lam = lam / Real(na);
+        Real uv[NP];
+        int m = 0;
 #pragma unroll
-        for (int a = 0; a < NP; ++a) out[a] = (act & (1u << a)) ? uv[m++] : Real(0);
-      }
+        for (int a = 0; a < NP; ++a)
+          if (act & (1u << a)) uv[m++] = ph[a] + P.mob_eps * (rate[a] - lam);
+        if (NP == 2) {
+          Real sv = uv[1];
+          sv = sv < Real(0) ? Real(0) : (sv > Real(1) ? Real(1) : sv);
+          out[1] = sv;
+          out[0] = Real(1) - sv;
+        } else {
+          project_simplex<Real, NP>(uv, m);
+          m = 0;
+#pragma unroll
+          for (int a = 0; a < NP; ++a) out[a] = (act & (1u << a)) ? uv[m++] : Real(0);
+        }
       }
     }
   }

@@ -58,16 +58,16 @@ struct Step3D {
   // fluxes alone (see pf_face; with shrinkage both, see pf_flux)
   static constexpr int NF = NP == 2 && !SHRINK ? 1 : NP;
   // resident CTAs per SM the register budget is cut for: two (64 registers)
-  // on D3Q19 in FP32, for any number of phases (three and four phases spill
-  // a few dozen bytes, yet two CTAs of 64 registers beat one of 128: 1.79
-  // against 1.91 ms on the ternary eutectic); FP64 and 27 populations: one
+  // on D3Q19 in FP32, for any number of phases (three and four phases spill 36
+  // to 138 bytes, yet two CTAs of 64 registers beat one of 128: 1.61 against
+  // 1.80 ms on the ternary eutectic); FP64 and 27 populations: one
   static constexpr int MIN_CTAS = (sizeof(Real) == 4 && QQ == 19) ? 2 : 1;
   // both paths in one launch where they have the same register budget and
   // the general path's shared memory is small (two phases: 37 KB).  A launch
   // reserves its largest path's shared memory for every CTA, and with more
-  // phases (96 KB) the liquid tiles are left too little L1 for their loads
-  // in flight: the ternary eutectic takes 1.88 ms a step in one launch,
-  // 1.77 ms in two.
+  // phases (74-96 KB) the liquid tiles are left too little L1 for their loads
+  // in flight: the ternary eutectic takes 1.78 ms a step in one launch,
+  // 1.61 ms in two.
   static constexpr bool ONE_LAUNCH = MIN_CTAS == 2 && NP == 2;
   static constexpr int OX = BX - 2, OY = BY - 2;
   static constexpr int W2 = BX + 2, H2 = BY + 2, C2 = W2 * H2;
@@ -531,46 +531,46 @@ __device__ __forceinline__ void general_tile(const DevParams<Real>& P, const Ste
       for (int a = 0; a < NF; ++a) pfz_hi[a] = Real(0);
     } else {
       if constexpr (DEFINITION) {
-      if (pfC) {
-        // in-plane faces of plane C into shared memory
-        Real fl[NP];
-        const bool cx_hi = P.bc[0] == kWall && (gx + 1 == 0 || gx + 1 == nx);
-        pf_flux(C, r2, C, r2 + 1, 0, cx_hi, fl);
+        if (pfC) {
+          // in-plane faces of plane C into shared memory
+          Real fl[NP];
+          const bool cx_hi = P.bc[0] == kWall && (gx + 1 == 0 || gx + 1 == nx);
+          pf_flux(C, r2, C, r2 + 1, 0, cx_hi, fl);
 #pragma unroll
-        for (int a = 0; a < NP; ++a) s_flux[a * (S::PFX + S::PFY) + ty * (BX + 1) + tx + 1] = fl[a];
-        // The first face of every row by the lanes of one warp (a lane of each
-        // row's own warp costs every warp a face: anisotropic eutectic
-        // 64 x 60 x 66 in FP32, 164 us a step, 154 so), but not where registers
-        // are short (shrinkage, dendrite 150 x 130 x 171: 312 us, 319 so; turned
-        // axes, eutectic 150 x 130 x 171: 657 us, 708 so).
-        constexpr bool OWN = SHRINK || EXT;
-        if (OWN ? tx == 0 : tid >= NT - BY) {
-          const int j = OWN ? ty : tid - (NT - BY), first = OWN ? gx : x0 - 1;
-          const bool cx_lo = P.bc[0] == kWall && (first == 0 || first == nx);
-          pf_flux(C, (j + 1) * W2, C, (j + 1) * W2 + 1, 0, cx_lo, fl);
+          for (int a = 0; a < NP; ++a) s_flux[a * (S::PFX + S::PFY) + ty * (BX + 1) + tx + 1] = fl[a];
+          // The first face of every row by the lanes of one warp (a lane of each
+          // row's own warp costs every warp a face: anisotropic eutectic
+          // 64 x 60 x 66 in FP32, 164 us a step, 154 so), but not where registers
+          // are short (shrinkage, dendrite 150 x 130 x 171: 312 us, 319 so; turned
+          // axes, eutectic 150 x 130 x 171: 657 us, 708 so).
+          constexpr bool OWN = SHRINK || EXT;
+          if (OWN ? tx == 0 : tid >= NT - BY) {
+            const int j = OWN ? ty : tid - (NT - BY), first = OWN ? gx : x0 - 1;
+            const bool cx_lo = P.bc[0] == kWall && (first == 0 || first == nx);
+            pf_flux(C, (j + 1) * W2, C, (j + 1) * W2 + 1, 0, cx_lo, fl);
 #pragma unroll
-          for (int a = 0; a < NP; ++a) s_flux[a * (S::PFX + S::PFY) + j * (BX + 1)] = fl[a];
+            for (int a = 0; a < NP; ++a) s_flux[a * (S::PFX + S::PFY) + j * (BX + 1)] = fl[a];
+          }
+          const bool cy_hi = P.bc[1] == kWall && (gy + 1 == 0 || gy + 1 == ny);
+          pf_flux(C, r2, C, r2 + W2, 1, cy_hi, fl);
+#pragma unroll
+          for (int a = 0; a < NP; ++a) s_flux[a * (S::PFX + S::PFY) + S::PFX + (ty + 1) * BX + tx] = fl[a];
+          if (ty == 0) {
+            const bool cy_lo = P.bc[1] == kWall && (gy == 0 || gy == ny);
+            pf_flux(C, r2 - W2, C, r2, 1, cy_lo, fl);
+#pragma unroll
+            for (int a = 0; a < NP; ++a) s_flux[a * (S::PFX + S::PFY) + S::PFX + tx] = fl[a];
+          }
         }
-        const bool cy_hi = P.bc[1] == kWall && (gy + 1 == 0 || gy + 1 == ny);
-        pf_flux(C, r2, C, r2 + W2, 1, cy_hi, fl);
-#pragma unroll
-        for (int a = 0; a < NP; ++a) s_flux[a * (S::PFX + S::PFY) + S::PFX + (ty + 1) * BX + tx] = fl[a];
-        if (ty == 0) {
-          const bool cy_lo = P.bc[1] == kWall && (gy == 0 || gy == ny);
-          pf_flux(C, r2 - W2, C, r2, 1, cy_lo, fl);
-#pragma unroll
-          for (int a = 0; a < NP; ++a) s_flux[a * (S::PFX + S::PFY) + S::PFX + tx] = fl[a];
+        // z-faces of this column: (C, C+1), and (C-1, C) on the first plane
+        if (pfC || below) {
+          const bool cz_hi = P.bc[2] == kWall && (C + 1 == 0 || C + 1 == nz);
+          pf_flux(C, r2, C + 1, r2, 2, cz_hi, pfz_hi);
+          if (SHRINK && C == z0 - 1) {
+            const bool cz_lo = P.bc[2] == kWall && (C == 0 || C == nz);
+            pf_flux(C - 1, r2, C, r2, 2, cz_lo, pfz_lo);
+          }
         }
-      }
-      // z-faces of this column: (C, C+1), and (C-1, C) on the first plane
-      if (pfC || below) {
-        const bool cz_hi = P.bc[2] == kWall && (C + 1 == 0 || C + 1 == nz);
-        pf_flux(C, r2, C + 1, r2, 2, cz_hi, pfz_hi);
-        if (SHRINK && C == z0 - 1) {
-          const bool cz_lo = P.bc[2] == kWall && (C == 0 || C == nz);
-          pf_flux(C - 1, r2, C, r2, 2, cz_lo, pfz_lo);
-        }
-      }
       } else if (pfC) {
         // f = 0: the first face of every row and column, by the lanes of two
         // warps; 1, 2: the +x and +y faces into shared memory; 3: the z-face
@@ -723,69 +723,69 @@ __device__ __forceinline__ void general_tile(const DevParams<Real>& P, const Ste
           out[1] = v;
           out[0] = Real(1) - v;
         } else {
-        Real ph[NP];
+          Real ph[NP];
 #pragma unroll
-        for (int a = 0; a < NP; ++a) ph[a] = out[a];
-        // central differences of phase a along axis t
-        auto grad = [&](int a, int t) -> Real {
-          return t == 0 ? Real(0.5) * (PH(C, a, r2 + 1) - PH(C, a, r2 - 1))
-                        : (t == 1 ? Real(0.5) * (PH(C, a, r2 + W2) - PH(C, a, r2 - W2))
-                                  : Real(0.5) * (PH(C + 1, a, r2) - PH(C - 1, a, r2)));
-        };
-        // the gradient energy's centre terms: dA/dq = 2 q, q_ab = phi_a g_b -
-        // phi_b g_a, by the products g_a . g_b
-        Real G[NP][NP], dadphi[NP];
+          for (int a = 0; a < NP; ++a) ph[a] = out[a];
+          // central differences of phase a along axis t
+          auto grad = [&](int a, int t) -> Real {
+            return t == 0 ? Real(0.5) * (PH(C, a, r2 + 1) - PH(C, a, r2 - 1))
+                          : (t == 1 ? Real(0.5) * (PH(C, a, r2 + W2) - PH(C, a, r2 - W2))
+                                    : Real(0.5) * (PH(C + 1, a, r2) - PH(C - 1, a, r2)));
+          };
+          // the gradient energy's centre terms: dA/dq = 2 q, q_ab = phi_a g_b -
+          // phi_b g_a, by the products g_a . g_b
+          Real G[NP][NP], dadphi[NP];
 #pragma unroll
-        for (int a = 0; a < NP; ++a) dadphi[a] = Real(0);
+          for (int a = 0; a < NP; ++a) dadphi[a] = Real(0);
 #pragma unroll
-        for (int t = 0; t < 3; ++t) {
-          Real g[NP];
+          for (int t = 0; t < 3; ++t) {
+            Real g[NP];
 #pragma unroll
-          for (int a = 0; a < NP; ++a) g[a] = grad(a, t);
+            for (int a = 0; a < NP; ++a) g[a] = grad(a, t);
+#pragma unroll
+            for (int a = 0; a < NP; ++a)
+#pragma unroll
+              for (int b = a; b < NP; ++b) G[a][b] = t == 0 ? g[a] * g[b] : G[a][b] + g[a] * g[b];
+          }
 #pragma unroll
           for (int a = 0; a < NP; ++a)
 #pragma unroll
-            for (int b = a; b < NP; ++b) G[a][b] = t == 0 ? g[a] * g[b] : G[a][b] + g[a] * g[b];
-        }
+            for (int b = a + 1; b < NP; ++b) {
+              const Real g2 = Real(2) * P.gamma[a][b];
+              dadphi[a] += g2 * (ph[a] * G[b][b] - ph[b] * G[a][b]);
+              dadphi[b] += g2 * (ph[b] * G[a][a] - ph[a] * G[a][b]);
+            }
+          Real psi[NP];
 #pragma unroll
-        for (int a = 0; a < NP; ++a)
+          for (int b = 0; b < NP; ++b) {
+            Real sv = P.S[b] * theta;
 #pragma unroll
-          for (int b = a + 1; b < NP; ++b) {
-            const Real g2 = Real(2) * P.gamma[a][b];
-            dadphi[a] += g2 * (ph[a] * G[b][b] - ph[b] * G[a][b]);
-            dadphi[b] += g2 * (ph[b] * G[a][a] - ph[a] * G[a][b]);
+            for (int i = 0; i < NC; ++i) sv -= mu[i] * mu[i] * P.inv4A[b] + mu[i] * ceq_of(b, i, fzC);
+            psi[b] = sv;
           }
-        Real psi[NP];
+          Real drv[NP];
+          driving_force<NP>(ph, psi, drv);
+          Real rate[NP], lam = Real(0);
+          int na = 0;
 #pragma unroll
-        for (int b = 0; b < NP; ++b) {
-          Real sv = P.S[b] * theta;
+          for (int a = 0; a < NP; ++a) {
+            Real obst = Real(0);
 #pragma unroll
-          for (int i = 0; i < NC; ++i) sv -= mu[i] * mu[i] * P.inv4A[b] + mu[i] * ceq_of(b, i, fzC);
-          psi[b] = sv;
-        }
-        Real drv[NP];
-        driving_force<NP>(ph, psi, drv);
-        Real rate[NP], lam = Real(0);
-        int na = 0;
-#pragma unroll
-        for (int a = 0; a < NP; ++a) {
-          Real obst = Real(0);
-#pragma unroll
-          for (int b = 0; b < NP; ++b)
-            if (b != a) obst += P.gamma[a][b] * ph[b];
-          const Real* fa = s_flux + a * (S::PFX + S::PFY);
-          const Real div = (fa[ty * (BX + 1) + tx + 1] - fa[ty * (BX + 1) + tx]) +
-                           (fa[S::PFX + (ty + 1) * BX + tx] - fa[S::PFX + ty * BX + tx]) + (pfz_hi[a] - pfz_lo[a]);
-          rate[a] = P.eps * (div - dadphi[a]) - P.obst * obst - drv[a];
-          if (act & (1u << a)) {
-            lam += rate[a];
-            ++na;
+            for (int b = 0; b < NP; ++b)
+              if (b != a) obst += P.gamma[a][b] * ph[b];
+            const Real* fa = s_flux + a * (S::PFX + S::PFY);
+            const Real div = (fa[ty * (BX + 1) + tx + 1] - fa[ty * (BX + 1) + tx]) +
+                             (fa[S::PFX + (ty + 1) * BX + tx] - fa[S::PFX + ty * BX + tx]) + (pfz_hi[a] - pfz_lo[a]);
+            rate[a] = P.eps * (div - dadphi[a]) - P.obst * obst - drv[a];
+            if (act & (1u << a)) {
+              lam += rate[a];
+              ++na;
+            }
           }
-        }
-        lam *= na == 2 ? Real(0.5) : (na == 3 ? Real(1.0 / 3.0) : Real(0.25));
+          lam *= na == 2 ? Real(0.5) : (na == 3 ? Real(1.0 / 3.0) : Real(0.25));
 #pragma unroll
-        for (int a = 0; a < NP; ++a) out[a] = ph[a] + P.mob_eps * (rate[a] - lam);
-        project_present<NP>(out, act);
+          for (int a = 0; a < NP; ++a) out[a] = ph[a] + P.mob_eps * (rate[a] - lam);
+          project_present<NP>(out, act);
         }
       }
     }

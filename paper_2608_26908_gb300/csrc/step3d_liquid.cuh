@@ -306,6 +306,8 @@ __global__ void __launch_bounds__(Step3D<NP, NC, Real, Store, QQ, SHRINK>::NT, S
   const int gxt = gridDim.x, gyt = gridDim.y, gzt = (P.v_hi - P.v_lo + ZS - 1) / ZS;
   const int bx = blockIdx.x, by = blockIdx.y;
   const bool liquid_pass = S::ONE_LAUNCH && (int)blockIdx.z >= gzt;
+  // (a shrinkage launch has no liquid pass; the kernel without its code is 3 %
+  // slower all the same, 322 against 313 us on the dendrite 150 x 130 x 171)
   if constexpr (S::ONE_LAUNCH) {
     if (liquid_pass) {
       liquid_tiles<NP, NC, Real, Store, QQ, EXT>(P, io, bx, by, ((int)blockIdx.z - gzt) * P.liq_group, gxt, gyt);
