@@ -671,11 +671,11 @@ gpflbm_status create_impl(const gpflbm_grid* grid, int n_phases, int n_component
     return GPFLBM_ERR_CUDA;
   }
   // Padding cells stay finite, and no tile is flagged liquid.  The memset runs
-  // on the legacy default stream, which non-blocking streams do not wait for
-  // and which does not wait for them: earlier work on the caller's workspace
-  // is let finish first, and the memset before the caller's first load.
-  e = cudaDeviceSynchronize();
-  if (e == cudaSuccess) e = cudaMemset(h->ws, 0, h->lay.total);
+  // on the legacy default stream, which non-blocking streams do not wait for:
+  // it is waited for here, before the caller's first load.  (That stream alone:
+  // waiting for the device would end another thread's stream capture, such as
+  // that of another handle's steps.)
+  e = cudaMemset(h->ws, 0, h->lay.total);
   if (e == cudaSuccess) e = cudaStreamSynchronize(nullptr);
   if (e != cudaSuccess) {
     std::fprintf(stderr, "gpflbm_create: %s\n", cudaGetErrorString(e));

@@ -60,3 +60,37 @@ def test_a_state_loaded_right_after_creation_stays():
         side.synchronize()
         assert torch.equal(got["phi"].reshape(-1), phi.reshape(-1))
         assert torch.equal(got["mu"].reshape(-1), mu.reshape(-1))
+
+
+def test_handles_created_while_another_thread_captures_steps():
+    """The steps' stream capture of one thread and the creation of handles in
+    another do not disturb each other."""
+    import threading
+
+    import torch
+
+    sc = inputs.scenario("dendrite2d", nx=64, ny=48, precision="fp32")
+    state = inputs.initial_state(sc)
+    errors, done = [], threading.Event()
+
+    def create():
+        try:
+            with torch.cuda.stream(torch.cuda.Stream()):
+                while not done.is_set():
+                    gpflbm.Sim(sc).close()
+        except Exception as e:  # noqa: BLE001 (reported by the main thread)
+            errors.append(e)
+
+    sim = gpflbm.Sim(sc)
+    sim.set_state(*state)
+    t = threading.Thread(target=create)
+    t.start()
+    try:
+        for _ in range(60):
+            sim.set_params(sc)  # drops the captured steps
+            sim.step(18)
+    finally:
+        done.set()
+        t.join()
+    assert not errors
+    torch.cuda.synchronize()
