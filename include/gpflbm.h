@@ -141,9 +141,10 @@ gpflbm_status gpflbm_workspace_bytes(const gpflbm_grid* grid, int n_phases, int 
  * memory of at least gpflbm_workspace_bytes() bytes, 256-byte aligned, owned
  * by the caller and kept alive (and untouched) until gpflbm_destroy; pass
  * NULL to let the library allocate (and later free) it with cudaMalloc.
- * No queued work may still use the workspace: the call clears it, and returns
- * once it is cleared.  The state is undefined until gpflbm_set_state.  On
- * failure *out is NULL. */
+ * The workspace is cleared on the legacy default stream, after what is queued
+ * there; no work queued elsewhere may still use it.  The state is undefined
+ * until gpflbm_set_state, whose stream waits for the clearing.  On failure *out
+ * is NULL. */
 gpflbm_status gpflbm_create(const gpflbm_grid* grid, int n_phases, int n_components,
                             const gpflbm_params* params, void* workspace, size_t workspace_bytes,
                             gpflbm_t* out);

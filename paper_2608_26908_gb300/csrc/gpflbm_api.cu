@@ -49,6 +49,7 @@ struct gpflbm_s {
   int cur;            // buffer holding the current state
   long long t;        // step counter of the current state
   bool has_state;
+  cudaEvent_t ev_clear;  // the workspace is cleared (until the first state is loaded)
   bool flags_stale;   // the liquid flags of both buffers await the next step (set_params)
   cudaStream_t capture;
   // adjoint: the stream that recomputes segments, and its events
@@ -672,11 +673,12 @@ gpflbm_status create_impl(const gpflbm_grid* grid, int n_phases, int n_component
   }
   // Padding cells stay finite, and no tile is flagged liquid.  The memset runs
   // on the legacy default stream, which non-blocking streams do not wait for:
-  // it is waited for here, before the caller's first load.  (That stream alone:
-  // waiting for the device would end another thread's stream capture, such as
-  // that of another handle's steps.)
+  // the first load waits for it (see set_state).  No wait on the host, which
+  // would hold the caller's queued work up, nor for the device, which would
+  // end another thread's stream capture.
   e = cudaMemset(h->ws, 0, h->lay.total);
-  if (e == cudaSuccess) e = cudaStreamSynchronize(nullptr);
+  if (e == cudaSuccess) e = cudaEventCreateWithFlags(&h->ev_clear, cudaEventDisableTiming);
+  if (e == cudaSuccess) e = cudaEventRecord(h->ev_clear, nullptr);
   if (e != cudaSuccess) {
     std::fprintf(stderr, "gpflbm_create: %s\n", cudaGetErrorString(e));
     gpflbm_destroy(h);
@@ -757,6 +759,13 @@ gpflbm_status gpflbm_set_state(gpflbm_t h, const void* phi, const void* mu, cons
   void* mu_d = own(h, h->lay.mu[h->cur], rs);
   void* f_d = own(h, h->lay.f[h->cur], ss);
   cudaError_t e;
+  if (h->ev_clear) {
+    // (a stream that is being captured cannot wait for work outside the capture)
+    cudaStreamCaptureStatus c = cudaStreamCaptureStatusNone;
+    e = cudaStreamIsCapturing(s, &c);
+    if (e == cudaSuccess && c == cudaStreamCaptureStatusNone) e = cudaStreamWaitEvent(s, h->ev_clear, 0);
+    if (e != cudaSuccess) return cuda_fail(h, e, "set_state: cleared workspace");
+  }
   bool staged = false;
   if (!on_device) {
     // pinned host sources are read by the load kernels in place
@@ -843,6 +852,8 @@ gpflbm_status gpflbm_set_state(gpflbm_t h, const void* phi, const void* mu, cons
     e = cudaStreamSynchronize(s);  // host sources must outlive the copies and loads
     if (e != cudaSuccess) return cuda_fail(h, e, "set_state: synchronize");
   }
+  if (h->ev_clear) cudaEventDestroy(h->ev_clear);
+  h->ev_clear = nullptr;
   h->t = t0;
   h->has_state = true;
   h->link_load = false;
@@ -1224,6 +1235,10 @@ const char* gpflbm_last_error(gpflbm_t h) { return h ? h->err.c_str() : "null ha
 void gpflbm_destroy(gpflbm_t h) {
   if (!h) return;
   drop_graphs(h);
+  if (h->ev_clear) {
+    cudaEventSynchronize(h->ev_clear);  // the caller may free the workspace once this returns
+    cudaEventDestroy(h->ev_clear);
+  }
   if (h->capture) cudaStreamDestroy(h->capture);
   if (h->xfer) {
     // an asynchronous load may still write the workspace, which the caller

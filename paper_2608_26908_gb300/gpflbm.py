@@ -202,9 +202,11 @@ class Sim:
                 raise GpflbmError(st, "gpflbm_slab_workspace_bytes")
             nbytes = n.value
         self.workspace = torch.empty(nbytes, dtype=torch.uint8, device="cuda")
-        # what torch queued on the block for its last owner ends before the
-        # library clears it
-        torch.cuda.current_stream().synchronize()
+        # the library clears the block on the default stream, after what torch
+        # queued here for its last owner
+        here, default = torch.cuda.current_stream(), torch.cuda.default_stream()
+        if here != default:
+            default.wait_stream(here)
         h = ctypes.c_void_p()
         if slab is None:
             st = lib().gpflbm_create(ctypes.byref(self._grid), self.NP, self.NC,

@@ -45,8 +45,8 @@ def test_parameters_changed_with_steps_in_flight(name):
 
 
 def test_a_state_loaded_right_after_creation_stays():
-    """The workspace is cleared before gpflbm_create returns: a load on a side
-    stream directly after it is not wiped."""
+    """A load on a side stream directly after gpflbm_create waits for the
+    clearing of the workspace and is not wiped by it."""
     import torch
 
     sc = inputs.scenario("eutectic3d", nx=256, ny=256, nz=128)
